@@ -45,8 +45,9 @@ extern "C" {
 #define PLAST_E_OOM (-2)      /* a device allocation failed */
 #define PLAST_E_CAPACITY (-3) /* output buffer too small; *n_out = needed */
 #define PLAST_E_CUDA (-4)     /* a CUDA runtime call or kernel failed */
-#define PLAST_E_TIMEOUT (-5)  /* a bounded device-side wait expired (reserved: no
-                                 kernel of this library waits on another CTA) */
+#define PLAST_E_TIMEOUT (-5)  /* a bounded device-side wait expired (the waits between the
+                                 warps of stage 2's tensor kernel; no kernel of this
+                                 library waits on another CTA) */
 
 #define PLAST_NKEYS 8800 /* subset-seed keys: 20 * 2 * 11 * 20 */
 #define PLAST_MAX_STAGES 5 /* stage intervals reported by plast_stage_times */
@@ -371,8 +372,8 @@ int plast_set_schedule(int mode);
 
 /*
  * Stage-2 tile shapes.  The work of a key is cut into tiles of consecutive
- * bank-1 occurrences: wide tiles of 128 rows, whose profile serves 4 bank-2
- * windows per warp, and narrow tiles of 16, 8, 4 or 2 rows, one bank-2
+ * bank-1 occurrences: wide tiles of up to 128 rows (on the tensor cores for
+ * thresholds s1 of 32 and more, by a packed int16 kernel below), and narrow tiles of 16, 8, 4 or 2 rows, one bank-2
  * window per lane, for short lists (a small query bank against a large one,
  * the end of a long list).  After the full wide tiles of a key, the library
  * covers the remainder either with one wide tile or with narrow tiles (16
@@ -381,11 +382,13 @@ int plast_set_schedule(int mode);
  * tile of shape S costs
  * S_slot x (rows of S) x ceil(n2 / P_S) x P_S + S_tile SM-nanoseconds, n2 the
  * key's bank-2 occurrences, P_S the bank-2 windows a CTA scores per pass
- * (128 wide, 512 narrow).  plast_autotune measures the constants on the
+ * (128 wide, 512 narrow).  (On the tensor cores a wide tile that is not full
+ * is charged (its rows rounded up to 32, plus 83) / 211 of the slots: a pass
+ * has a fixed part worth 83 rows.)  plast_autotune measures the constants on the
  * current device (random banks, the stage-2 kernel timed with every tile of
  * one shape, against a long and a short bank 2; about a second), installs
- * them and copies them to *out (may be NULL).  It also picks the wide kernel
- * variant by timing each: how many cells of the wide profile are held as
+ * them and copies them to *out (may be NULL).  It also picks the variant of
+ * the packed int16 wide kernel by timing each: how many cells of the wide profile are held as
  * int16 (no sign extension, twice the shared-memory traffic), then how many
  * passes ahead a warp fetches its next bank-2 windows (the staging depth).
  * plast_get_tile_costs / plast_set_tile_costs read and install costs and
@@ -410,8 +413,8 @@ int plast_get_tile_costs(plast_tile_costs* out);
 int plast_set_tile_costs(const plast_tile_costs* costs);
 int plast_set_tile_shape(int mode);
 /*
- * The stage-2 work list the library would run for two banks with the given
- * CSR key offsets (host arrays of PLAST_NKEYS + 1 entries each, as
+ * The stage-2 work list, every wide tile charged as a full one, of two banks with
+ * the given CSR key offsets (host arrays of PLAST_NKEYS + 1 entries each, as
  * plast_bank_export_index returns) on a GPU of n_sms SMs (0: no splitting of
  * long lists): host-only, no device needed.  Fills tiles[6 * t ..] with (key,
  * first bank-1 CSR index, rows, shape: 0 wide, 1, 2, 3, 4 narrow of 8, 4, 2,

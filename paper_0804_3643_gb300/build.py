@@ -4,7 +4,7 @@
 
 Each .cu file under csrc/ is compiled in parallel with one -gencode
 (compute_103a -> sm_103a), relocatable device code (the score tables live in
-constant memory shared across files), then linked into a shared library next
+constant memory shared across files; the files in WHOLE stand alone), then linked into a shared library next
 to this file.  Objects go to csrc/_build/ (git-ignored).
 """
 from __future__ import annotations
@@ -19,7 +19,10 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(CSRC, "_build")
 LIB = os.path.join(HERE, "libplast.so")
-SOURCES = ["prims.cu", "index.cu", "ungapped.cu", "filter.cu", "gapped.cu", "full.cu", "api.cu", "noalloc.cu"]
+SOURCES = ["prims.cu", "index.cu", "ungapped.cu", "ungapped_mma.cu", "filter.cu", "gapped.cu", "full.cu", "api.cu", "noalloc.cu"]
+# compiled as a whole program: it splits its registers with setmaxnreg, which
+# relocatable device code ignores
+WHOLE = {"ungapped_mma.cu"}
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -30,8 +33,9 @@ def nvcc() -> str:
     raise RuntimeError("nvcc not found")
 
 
-def _flags(verbose: bool):
-    f = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-rdc=true", "-Xcompiler", "-fPIC,-O2",
+def _flags(verbose: bool, src: str):
+    rdc = "-rdc=false" if os.path.basename(src) in WHOLE else "-rdc=true"
+    f = ARCH + ["-O3", "-lineinfo", "-std=c++17", rdc, "-Xcompiler", "-fPIC,-O2",
                 "-I" + os.path.join(HERE, "..", "include")]
     if verbose:
         f += ["-Xptxas", "-v"]
@@ -59,7 +63,7 @@ def build(verbose: bool = False, force: bool = False) -> str:
 
     def compile_one(job):
         src, obj = job
-        cmd = [cc] + _flags(verbose) + ["-c", src, "-o", obj]
+        cmd = [cc] + _flags(verbose, src) + ["-c", src, "-o", obj]
         r = subprocess.run(cmd, capture_output=True, text=True)
         return src, r
 

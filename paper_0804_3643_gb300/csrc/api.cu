@@ -144,12 +144,18 @@ int num_sms() {
 // tile.  A CTA moves through a key's bank-2 windows a pass at a time (32 warps
 // x 4 windows wide, x 32 narrow), so a tile is charged its shape's rows x n2
 // rounded up to that granularity.  Defaults from a GB300; plast_autotune
-// measures them on the current device.
+// measures them on the current device.  The wide costs are the tensor
+// kernel's, whose pass costs (rows rounded up to 32) + TC_FIXED_ROWS (measured:
+// 1.23, 1.5, 2.0 and 2.29 SM-microseconds a pass of 32, 64, 96 and 128 rows);
+// the plain wide kernel, which runs at an S1 below UNG_TC_MIN_S1, is charged
+// PLAIN_WIDE_SLOT for every row of the shape.
+constexpr int TC_FIXED_ROWS = 83;
+constexpr double PLAIN_WIDE_SLOT = 0.317, PLAIN_WIDE_TILE = 2960.0;
 std::mutex g_cost_mu;
-plast_tile_costs g_costs = {0.317, 2960.0, 0.479, 566.0, 0.616, 1101.0, 1.094, 1090.0, 12, 0, 0.416, 314.0};
+plast_tile_costs g_costs = {0.140, 3660.0, 0.479, 566.0, 0.616, 1101.0, 1.094, 1090.0, 12, 0, 0.416, 314.0};
 // 0: by cost; 1: wide only; 2, 3, 4, 5: narrow tiles of 8, 4, 2, 16 rows only
 std::atomic<int> g_shape{0};
-constexpr int64_t WIDE_PASS = (UNG_THREADS / 32) * 4;     // bank-2 windows per CTA pass, wide tile
+constexpr int64_t WIDE_PASS = 128;                         // bank-2 windows per CTA pass, wide tile
 constexpr int64_t NARROW_PASS = UNG_NARROW_PASS;           // narrow tiles
 int64_t round_up(int64_t n, int64_t g) { return (n + g - 1) / g * g; }
 
@@ -168,12 +174,16 @@ int shape_rows(int shape) {
   }
 }
 
-double shape_slots(int shape, int64_t n2) {
-  return (double)shape_rows(shape) * (double)round_up(n2, shape == UNG_WIDE ? WIDE_PASS : NARROW_PASS);
+// Slots a tile is charged for; rows: of a wide tile of the tensor kernel, the
+// rows it holds (a full tile's share of what its passes cost).
+double shape_slots(int shape, int64_t n2, int64_t rows = UNG_T1) {
+  const double full = (double)shape_rows(shape) * (double)round_up(n2, shape == UNG_WIDE ? WIDE_PASS : NARROW_PASS);
+  if (shape != UNG_WIDE || rows == UNG_T1) return full;
+  return full * (double)(round_up(rows, 32) + TC_FIXED_ROWS) / (double)(UNG_T1 + TC_FIXED_ROWS);
 }
 
-double tile_cost(const plast_tile_costs& c, int shape, int64_t n2) {
-  const double slots = shape_slots(shape, n2);
+double tile_cost(const plast_tile_costs& c, int shape, int64_t n2, int64_t rows = UNG_T1) {
+  const double slots = shape_slots(shape, n2, rows);
   switch (shape) {
     case UNG_WIDE:
       return c.wide_slot * slots + c.wide_tile;
@@ -198,25 +208,35 @@ struct TileList {
   std::vector<int4> tiles;        // (key, first CSR index of bank 1, rows, shape)
   int64_t n_wide = 0;             // persistent order: the wide tiles come first
   int64_t pairs = 0;
+  bool tensor = false;            // the wide tiles are the tensor kernel's
 };
+
+// The rows a tile is charged for: a partial wide tile of the tensor kernel
+// costs less than a full one.
+int64_t charged_rows(const int4& t, bool tensor) {
+  return tensor && tile_shape(t) == UNG_WIDE ? tile_rows(t) : UNG_T1;
+}
 
 // When a launch has too few tiles to keep its CTAs busy to the end (a small
 // query bank: a few hundred keys with one or two bank-1 occurrences), the
 // costliest tiles are cut along their bank-2 lists into pieces of whole
 // passes, so that no piece costs more than about 1/4 of a CTA's share; the
 // pieces re-sorted costliest first.  v[lo, hi) is one launch's tile list.
-void split_long_tiles(const plast_tile_costs& c, std::vector<int4>& v, int64_t lo, int64_t hi, int64_t ctas) {
+void split_long_tiles(const plast_tile_costs& c, std::vector<int4>& v, int64_t lo, int64_t hi, int64_t ctas,
+                      bool tensor) {
   if (hi <= lo || ctas <= 0) return;
+  auto cost = [&](const int4& t) {
+    return tile_cost(c, tile_shape(t), (int64_t)t.w - t.z, charged_rows(t, tensor));
+  };
   // the list is costliest first: a tile above twice the target exists only if
   // the first one is above it, and the target is at most the first tile's
   // cost times the tile count over 4 * ctas
   if (hi - lo > 8 * ctas) {
-    const double c0 = tile_cost(c, tile_shape(v[lo]), (int64_t)v[lo].w - v[lo].z);
+    const double c0 = cost(v[lo]);
     double total = 0;
-    for (int64_t i = lo; i < hi; i++) total += tile_cost(c, tile_shape(v[i]), (int64_t)v[i].w - v[i].z);
+    for (int64_t i = lo; i < hi; i++) total += cost(v[i]);
     if (c0 <= 2 * total / (4.0 * (double)ctas)) return;
   }
-  auto cost = [&](const int4& t) { return tile_cost(c, tile_shape(t), (int64_t)t.w - t.z); };
   double total = 0;
   for (int64_t i = lo; i < hi; i++) total += cost(v[i]);
   const double target = total / (4.0 * (double)ctas);
@@ -251,14 +271,19 @@ void split_long_tiles(const plast_tile_costs& c, std::vector<int4>& v, int64_t l
 }
 
 void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first, TileList* tl,
-                      const std::vector<char>* key_mask, int shape_override, int n_sms) {
+                      const std::vector<char>* key_mask, int shape_override, int n_sms, bool tensor, bool listed = false) {
   tl->tiles.clear();
+  tl->tensor = tensor;
   tl->pairs = 0;
   tl->n_wide = 0;
   plast_tile_costs c;
   {
     std::lock_guard<std::mutex> lk(g_cost_mu);
     c = g_costs;
+  }
+  if (!tensor && !listed) {
+    c.wide_slot = PLAIN_WIDE_SLOT;
+    c.wide_tile = PLAIN_WIDE_TILE;
   }
   const int mode = shape_override >= 0 ? shape_override : g_shape.load();
   // Keys in launch order: the persistent schedule takes them by decreasing
@@ -360,7 +385,7 @@ void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first
     const int64_t full = rem / br;
     const int tail = (int)(rem % br);
     const double narrow_cost = (double)full * cost_now[bulk] + best[tail];
-    if (!(narrow_cost < tile_cost(c, UNG_WIDE, n2))) {
+    if (!(narrow_cost < tile_cost(c, UNG_WIDE, n2, tensor ? rem : UNG_T1))) {
       emit(k, u, rem, UNG_WIDE);
       continue;
     }
@@ -398,8 +423,8 @@ void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first
   if (n_sms > 0) {
     std::vector<int4> wide(tl->tiles.begin(), tl->tiles.begin() + tl->n_wide);
     std::vector<int4> narrow(tl->tiles.begin() + tl->n_wide, tl->tiles.end());
-    split_long_tiles(c, wide, 0, (int64_t)wide.size(), (int64_t)n_sms);
-    split_long_tiles(c, narrow, 0, (int64_t)narrow.size(), (int64_t)UNG_NARROW_CTAS_PER_SM * n_sms);
+    split_long_tiles(c, wide, 0, (int64_t)wide.size(), (int64_t)n_sms, tensor);
+    split_long_tiles(c, narrow, 0, (int64_t)narrow.size(), (int64_t)UNG_NARROW_CTAS_PER_SM * n_sms, tensor);
     tl->tiles.assign(wide.begin(), wide.end());
     tl->n_wide = (int64_t)wide.size();
     tl->tiles.insert(tl->tiles.end(), narrow.begin(), narrow.end());
@@ -421,6 +446,7 @@ cudaError_t launch_tiles(const TileList& tl, UngArgs a, int32_t* counters, bool 
     a.persistent = persistent ? 1 : 0;
     const int per_sm = wide ? 1 : UNG_NARROW_CTAS_PER_SM;
     const int grid = persistent ? (int)std::min<int64_t>((int64_t)per_sm * num_sms(), hi - lo) : (int)(hi - lo);
+    if (wide && tl.tensor) return launch_ungapped_mma(a, grid, st);
     return wide ? launch_ungapped(a, grid, st) : launch_ungapped_narrow(a, grid, st);
   };
   if (persistent) {
@@ -441,11 +467,17 @@ cudaError_t launch_tiles(const TileList& tl, UngArgs a, int32_t* counters, bool 
   return cudaSuccess;
 }
 
-void build_tiles(const plast_bank* b1, const plast_bank* b2, bool largest_first, TileList* tl,
+// tensor: the wide tiles go to the tensor kernel (stage2_on_tensor), else to
+// the plain one.
+void build_tiles(const plast_bank* b1, const plast_bank* b2, bool largest_first, TileList* tl, bool tensor,
                  const std::vector<char>* key_mask = nullptr, int shape_override = -1) {
   build_tiles_from(b1->h_key_off.data(), b2->h_key_off.data(), largest_first, tl, key_mask, shape_override,
-                   largest_first ? num_sms() : 0);
+                   largest_first ? num_sms() : 0, tensor);
 }
+
+// The tensor kernel extends the pairs its bound lets through, so it pays at
+// thresholds that few pairs reach.
+bool stage2_on_tensor(const plast_params& prm) { return prm.s1 >= UNG_TC_MIN_S1; }
 
 // The survivor rate of the last stage 2 of each pair of banks, to size the
 // next one's survivor buffer.  The first guess, pairs / 128, holds for
@@ -503,7 +535,7 @@ int run_ungapped(const plast_bank* b1, const plast_bank* b2, const plast_params&
   sv->sh = b2->pad_bits;
   TileList tl;
   const int mode = g_schedule.load();
-  build_tiles(b1, b2, mode == 0, &tl, key_mask);
+  build_tiles(b1, b2, mode == 0, &tl, stage2_on_tensor(prm), key_mask);
   t_timer.mark(0, st);
   if (tl.tiles.empty()) return PLAST_OK;
   const int64_t nt = (int64_t)tl.tiles.size();
@@ -514,7 +546,7 @@ int run_ungapped(const plast_bank* b1, const plast_bank* b2, const plast_params&
   unsigned long long* d_count;
   CK(sc.get(&d_tiles, nt));
   CK(sc.get(&d_counter, 2));
-  CK(sc.get(&d_count, 1));
+  CK(sc.get(&d_count, 2));  // the survivors, then the kernels' error flag
   CK(cudaMemcpyAsync(d_tiles, tl.tiles.data(), nt * sizeof(int4), cudaMemcpyHostToDevice, st));
 
   int64_t cap = tl.pairs / 128 + (1 << 20);
@@ -526,7 +558,7 @@ int run_ungapped(const plast_bank* b1, const plast_bank* b2, const plast_params&
     CK(sc.get(&k0, cap));
     CK(sc.get(&v0, cap));
     CK(cudaMemsetAsync(d_counter, 0, 2 * sizeof(int32_t), st));
-    CK(cudaMemsetAsync(d_count, 0, sizeof(unsigned long long), st));
+    CK(cudaMemsetAsync(d_count, 0, 2 * sizeof(unsigned long long), st));
     UngArgs a;
     a.nb1 = b1->nb;
     a.pos1 = b1->pos;
@@ -541,12 +573,15 @@ int run_ungapped(const plast_bank* b1, const plast_bank* b2, const plast_params&
     a.out_count = d_count;
     a.cap = cap;
     a.sh = sv->sh;
+    a.err = reinterpret_cast<int32_t*>(d_count + 1);
     t_timer.mark(1, st);
     CK(launch_tiles(tl, a, d_counter, mode == 0, st));
     t_timer.mark(2, st);
-    unsigned long long n = 0;
-    CK(cudaMemcpyAsync(&n, d_count, sizeof(n), cudaMemcpyDeviceToHost, st));
+    unsigned long long h_count[2] = {0, 0};
+    CK(cudaMemcpyAsync(h_count, d_count, sizeof(h_count), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
+    if (h_count[1]) return PLAST_E_TIMEOUT;
+    unsigned long long n = h_count[0];
     if (tl.pairs > 0) set_rate_hint(b1, b2, (double)n / (double)tl.pairs);
     if ((int64_t)n > cap) {
       sc.release(k0);
@@ -1220,7 +1255,7 @@ struct plast_plan {
   int sh = 0, bits = 0;
   int4* tiles = nullptr;
   int32_t* counter = nullptr;
-  unsigned long long* count = nullptr;
+  unsigned long long* count = nullptr;  // stage-2 hits, then the kernels' error flag
   int64_t* n_dev = nullptr;   // survivors, clamped to max_hits
   int64_t* m_dev = nullptr;   // records, clamped to max_records
   uint64_t* k0 = nullptr;     // survivors (kernel order)
@@ -1285,14 +1320,14 @@ int plast_plan_create(const plast_bank* b1, const plast_bank* b2, const plast_pa
     return rc_of(e);
   };
   TileList& tl = p->tl;
-  build_tiles(b1, b2, true, &tl);
+  build_tiles(b1, b2, true, &tl, stage2_on_tensor(p->prm));
   p->n_tiles = (int64_t)tl.tiles.size();
   cudaError_t e;
   auto alloc = [&](void** q, size_t bytes) { return dev_alloc(q, bytes < 16 ? 16 : bytes); };
   p->rtb = radix_tmp_bytes(max_records);
   if ((e = alloc((void**)&p->tiles, sizeof(int4) * (size_t)std::max<int64_t>(p->n_tiles, 1))) ||
       (e = alloc((void**)&p->counter, 2 * sizeof(int32_t))) ||
-      (e = alloc((void**)&p->count, sizeof(unsigned long long))) ||
+      (e = alloc((void**)&p->count, 2 * sizeof(unsigned long long))) ||
       (e = alloc((void**)&p->n_dev, sizeof(int64_t))) || (e = alloc((void**)&p->m_dev, sizeof(int64_t))) ||
       (e = alloc((void**)&p->k0, 8 * (size_t)max_hits)) || (e = alloc((void**)&p->v0, 4 * (size_t)max_hits)) ||
       (e = alloc((void**)&p->rk0, 8 * (size_t)max_records)) || (e = alloc((void**)&p->rk1, 8 * (size_t)max_records)) ||
@@ -1314,6 +1349,7 @@ int plast_plan_create(const plast_bank* b1, const plast_bank* b2, const plast_pa
   GapArgs gnone{};
   gnone.n = 0;
   if ((e = launch_ungapped(none, 0, st)) || (e = launch_ungapped_narrow(none, 0, st)) ||
+      (e = launch_ungapped_mma(none, 0, st)) ||
       (e = launch_small_gapped(gnone, st)))
     return fail(e);
   if ((e = cudaStreamSynchronize(st))) return fail(e);
@@ -1326,7 +1362,7 @@ int plast_plan_run(plast_plan* p, void* stream) {
   if (!p) return PLAST_E_INVALID;
   cudaStream_t st = (cudaStream_t)stream;
   CK(cudaMemsetAsync(p->counter, 0, 2 * sizeof(int32_t), st));
-  CK(cudaMemsetAsync(p->count, 0, sizeof(unsigned long long), st));
+  CK(cudaMemsetAsync(p->count, 0, 2 * sizeof(unsigned long long), st));
   CK(cudaMemsetAsync(p->total, 0, sizeof(int64_t), st));
   if (p->n_tiles > 0) {
     UngArgs a;
@@ -1346,6 +1382,7 @@ int plast_plan_run(plast_plan* p, void* stream) {
     a.out_count = p->count;
     a.cap = p->max_hits;
     a.sh = p->sh;
+    a.err = reinterpret_cast<int32_t*>(p->count + 1);
     CK(launch_tiles(p->tl, a, p->counter, true, st));
   }
   CK(launch_clamp_count(p->count, p->max_hits, p->n_dev, st));
@@ -1418,12 +1455,14 @@ int plast_plan_launch(plast_plan* p, void* stream) {
 int plast_plan_result(const plast_plan* p, int64_t* n_records, int64_t* n_hits, void* stream) {
   if (!p || !n_records) return PLAST_E_INVALID;
   cudaStream_t st = (cudaStream_t)stream;
-  unsigned long long hits = 0, kept = 0;
+  unsigned long long count[2] = {0, 0}, kept = 0;
   int64_t recs = 0;
-  CK(cudaMemcpyAsync(&hits, p->count, sizeof(hits), cudaMemcpyDeviceToHost, st));
+  CK(cudaMemcpyAsync(count, p->count, sizeof(count), cudaMemcpyDeviceToHost, st));
   if (p->count_f) CK(cudaMemcpyAsync(&kept, p->count_f, sizeof(kept), cudaMemcpyDeviceToHost, st));
   CK(cudaMemcpyAsync(&recs, p->total, sizeof(recs), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
+  if (count[1]) return PLAST_E_TIMEOUT;
+  const unsigned long long hits = count[0];
   if (n_hits) *n_hits = (int64_t)(p->count_f && hits <= (unsigned long long)p->max_hits ? kept : hits);
   if ((int64_t)hits > p->max_hits) {
     *n_records = (int64_t)hits;
@@ -1473,16 +1512,16 @@ int random_bank(int32_t n_seqs, int len, uint64_t seed, cudaStream_t st, plast_b
 }
 
 // median device time (ms) of the stage-2 kernel over `reps` runs of the
-// given shape; *slots = sum over tiles of the charged slots, *tiles = count
-int time_stage2(const plast_bank* b1, const plast_bank* b2, int shape, cudaStream_t st, int reps, double* ms,
-                double* slots, double* tiles) {
+// given shape (tensor: wide tiles on the tensor kernel); *slots = sum over tiles of the charged slots, *tiles = count
+int time_stage2(const plast_bank* b1, const plast_bank* b2, int shape, bool tensor, cudaStream_t st, int reps,
+                double* ms, double* slots, double* tiles) {
   TileList tl;
   CK(bank_wait(b1, st));
   CK(bank_wait(b2, st));
-  build_tiles(b1, b2, true, &tl, nullptr, shape);
+  build_tiles(b1, b2, true, &tl, tensor, nullptr, shape);
   *slots = 0;
   for (const int4& t : tl.tiles) {
-    *slots += shape_slots(tile_shape(t), (int64_t)t.w - t.z);
+    *slots += shape_slots(tile_shape(t), (int64_t)t.w - t.z, charged_rows(t, tensor));
   }
   *tiles = (double)tl.tiles.size();
   *ms = 0;
@@ -1496,7 +1535,7 @@ int time_stage2(const plast_bank* b1, const plast_bank* b2, int shape, cudaStrea
   const int64_t cap = tl.pairs / 64 + (1 << 16);
   CK(sc.get(&d_tiles, tl.tiles.size()));
   CK(sc.get(&d_counter, 2));
-  CK(sc.get(&d_count, 1));
+  CK(sc.get(&d_count, 2));
   CK(sc.get(&k0, cap));
   CK(sc.get(&v0, cap));
   CK(cudaMemcpyAsync(d_tiles, tl.tiles.data(), tl.tiles.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
@@ -1519,6 +1558,7 @@ int time_stage2(const plast_bank* b1, const plast_bank* b2, int shape, cudaStrea
   a.out_count = d_count;
   a.cap = cap;
   a.sh = b2->pad_bits;
+  a.err = reinterpret_cast<int32_t*>(d_count + 1);
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0));
   if (cudaEventCreate(&e1) != cudaSuccess) {
@@ -1529,7 +1569,7 @@ int time_stage2(const plast_bank* b1, const plast_bank* b2, int shape, cudaStrea
   cudaError_t e = cudaSuccess;
   for (int r = 0; r <= reps && e == cudaSuccess; r++) {
     e = cudaMemsetAsync(d_counter, 0, 2 * sizeof(int32_t), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d_count, 0, sizeof(unsigned long long), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(d_count, 0, 2 * sizeof(unsigned long long), st);
     if (e == cudaSuccess) e = cudaEventRecord(e0, st);
     if (e == cudaSuccess) e = launch_tiles(tl, a, d_counter, true, st);
     if (e == cudaSuccess) e = cudaEventRecord(e1, st);
@@ -1586,7 +1626,7 @@ int plast_stage2_tiles(const int64_t* key_off1, const int64_t* key_off2, int32_t
       return PLAST_E_INVALID;
   TileList tl;
   const bool persistent = g_schedule.load() == 0;
-  build_tiles_from(key_off1, key_off2, persistent, &tl, nullptr, -1, persistent ? n_sms : 0);
+  build_tiles_from(key_off1, key_off2, persistent, &tl, nullptr, -1, persistent ? n_sms : 0, false, true);
   *n_tiles = (int64_t)tl.tiles.size();
   if (*n_tiles > cap) return PLAST_E_CAPACITY;
   for (size_t i = 0; i < tl.tiles.size(); i++) {
@@ -1611,20 +1651,23 @@ int plast_set_tile_shape(int mode) {
 int plast_autotune(void* stream, plast_tile_costs* out) {
   cudaStream_t st = (cudaStream_t)stream;
   CK(upload_tables_once());
-  plast_bank *b1 = nullptr, *b2l = nullptr, *b2s = nullptr;
-  // bank 1: ~10 occurrences per key; bank 2: ~4,100 (four narrow passes)
-  // and ~300 (two wide passes, a fraction of a narrow one) per key
+  plast_bank *b1 = nullptr, *b1w = nullptr, *b2l = nullptr, *b2s = nullptr;
+  // bank 1: ~10 occurrences per key (narrow), ~110 (wide); bank 2: ~4,100
+  // (four narrow passes) and ~300 (two wide passes, a fraction of a narrow
+  // one) per key
   int rc = random_bank(300, 300, 11, st, &b1);
+  if (rc == PLAST_OK) rc = random_bank(3300, 300, 14, st, &b1w);
   if (rc == PLAST_OK) rc = random_bank(120000, 300, 12, st, &b2l);
   if (rc == PLAST_OK) rc = random_bank(9000, 300, 13, st, &b2s);
   plast_tile_costs c;
   plast_get_tile_costs(&c);
   const double sms = (double)num_sms();
   // slot and tile cost of a shape from its times on the long and short bank 2
-  auto fit = [&](int shape, double* slot, double* tile, double* t_long) {
+  auto fit = [&](int shape, bool tensor, double* slot, double* tile, double* t_long) {
     double t_l, s_l, n_l, t_s, s_s, n_s;
-    int r = time_stage2(b1, b2l, shape, st, 3, &t_l, &s_l, &n_l);
-    if (r == PLAST_OK) r = time_stage2(b1, b2s, shape, st, 3, &t_s, &s_s, &n_s);
+    const plast_bank* q = tensor ? b1w : b1;
+    int r = time_stage2(q, b2l, shape, tensor, st, 3, &t_l, &s_l, &n_l);
+    if (r == PLAST_OK) r = time_stage2(q, b2s, shape, tensor, st, 3, &t_s, &s_s, &n_s);
     if (r != PLAST_OK) return r;
     // SM-nanoseconds = slot cost x slots + tile cost x tiles, for both banks
     const double y_l = t_l * 1e6 * sms, y_s = t_s * 1e6 * sms;
@@ -1641,16 +1684,15 @@ int plast_autotune(void* stream, plast_tile_costs* out) {
   const int saved_variant = ungapped_variant();
   double best_t = 0;
   int best_v = saved_variant;
-  // the int16 cells at staging depth 1, then the staging depths of the best
+  // the plain wide kernel's variant: the int16 cells at staging depth 1, then
+  // the staging depths of the best
   auto try_variant = [&](int v, bool first) {
     set_ungapped_variant(v);
     double slot, tile, t_long;
-    rc = fit(1, &slot, &tile, &t_long);
+    rc = fit(1, false, &slot, &tile, &t_long);
     if (rc == PLAST_OK && (first || t_long < best_t)) {
       best_t = t_long;
       best_v = v;
-      c.wide_slot = slot;
-      c.wide_tile = tile;
       c.wide_int16_cells = ungapped_variant_n16(v);
       c.wide_stage_depth = ungapped_variant_depth(v);
     }
@@ -1661,11 +1703,13 @@ int plast_autotune(void* stream, plast_tile_costs* out) {
     try_variant(v, false);
   set_ungapped_variant(rc == PLAST_OK ? best_v : saved_variant);
   double t_long;
-  if (rc == PLAST_OK) rc = fit(2, &c.narrow_slot, &c.narrow_tile, &t_long);
-  if (rc == PLAST_OK) rc = fit(3, &c.narrow4_slot, &c.narrow4_tile, &t_long);
-  if (rc == PLAST_OK) rc = fit(4, &c.narrow2_slot, &c.narrow2_tile, &t_long);
-  if (rc == PLAST_OK) rc = fit(5, &c.narrow16_slot, &c.narrow16_tile, &t_long);
+  if (rc == PLAST_OK) rc = fit(1, true, &c.wide_slot, &c.wide_tile, &t_long);
+  if (rc == PLAST_OK) rc = fit(2, false, &c.narrow_slot, &c.narrow_tile, &t_long);
+  if (rc == PLAST_OK) rc = fit(3, false, &c.narrow4_slot, &c.narrow4_tile, &t_long);
+  if (rc == PLAST_OK) rc = fit(4, false, &c.narrow2_slot, &c.narrow2_tile, &t_long);
+  if (rc == PLAST_OK) rc = fit(5, false, &c.narrow16_slot, &c.narrow16_tile, &t_long);
   plast_bank_free(b1);
+  plast_bank_free(b1w);
   plast_bank_free(b2l);
   plast_bank_free(b2s);
   if (rc != PLAST_OK) return rc;

@@ -39,6 +39,7 @@ struct UngArgs {
   unsigned long long* out_count;
   int64_t cap;              // capacity of out_key / out_val
   int32_t sh;               // bits of a bank-2 padded position
+  int32_t* err;             // raised when a bounded wait of the tensor kernel ran out
 };
 
 // Wide-tile variants of the stage-2 kernel: how many cells the profile holds
@@ -54,6 +55,13 @@ void set_ungapped_variant(int v);    // -1: the default
 // wide tiles (the current variant) / narrow tiles, each a persistent launch
 cudaError_t launch_ungapped(const UngArgs& a, int grid, cudaStream_t st);
 cudaError_t launch_ungapped_narrow(const UngArgs& a, int grid, cudaStream_t st);
+cudaError_t launch_ungapped_mma(const UngArgs& a, int grid, cudaStream_t st);
+constexpr int UNG_TC_PASS = 128;      // bank-2 windows the tensor kernel scores per pass
+// Lowest S1 whose wide tiles go to the tensor kernel: below it more pairs pass
+// the bound than their exact extension is worth (3,000 x 20,000 proteins, ms:
+// S1 = 38 1.81 against the plain kernel's 3.36, 34 2.54 / 3.50, 32 3.45 / 3.58,
+// 30 4.75 / 3.68).
+constexpr int UNG_TC_MIN_S1 = 32;
 constexpr int UNG_NARROW_CTAS_PER_SM = 2;
 constexpr int UNG_NARROW_PASS = 512;  // bank-2 windows a narrow CTA scores per pass
 }  // namespace plast
