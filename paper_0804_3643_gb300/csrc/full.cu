@@ -13,7 +13,7 @@
 // One side of one record is an anchored dynamic programme without a band,
 // cut by the drop-off X row by row: a cell whose H is more than X below T,
 // the best H of the rows before it, is dropped (H = F = minus infinity).  The
-// warp computes a row 32 columns at a time, one column per lane, from the
+// warp computes a row 64 columns at a time, two columns per lane, from the
 // first live column of the row above:
 //   F  = max(F_up - ge, H_up - go - ge)        (shared memory: the row above)
 //   D  = H_diag + s(A_i, B_j)
@@ -81,27 +81,65 @@ constexpr int FG_SLOTS = FG_W + 4;  // the row buffer: two dead slots before the
 // offset, line, stored columns per row) are in `arena`.  *err gets FG_ERR_*
 // bits on a capacity overflow.
 //
-// A row is computed 64 columns at a time, two adjacent columns j0 = cs + 2l
-// and j0 + 1 per lane, from an even origin o at or left of the row's first
-// column c0 (the column left of c0 that the rounding may add comes out
-// dead and is not counted), so that a row of the random extensions (about
-// 40 columns) takes one pass and one scan.  Column j is kept in slot
-// j - o + 2 (slots 0 and 1 hold the dead value), so the two slots a lane
-// reads and writes are one aligned 8-byte word; the E scan runs over the
-// lanes' pairwise maxima.  Values are computed relative to the line of the
-// row above (the stored int16 decode with no add), the live test and the
-// stored values relative to the row's own line.  Each lane keeps, over the
-// row's chunks, its first and last live column and its best key (H - line)
-// << 11 | (2047 - (j - o)) of a live cell; three warp reductions at the
-// row's end give the live window, the row maximum and its first column.
+// A row is computed 64 columns at a time, two adjacent columns per lane, from
+// an even origin o at or left of the row's first column c0 (the column left of
+// c0 that the rounding may add comes out dead and is not counted).  A row that
+// ends within its first 64 columns (nearly all of them at the usual drop-offs:
+// a cell further than (X + 11 - go) / ge columns from its best is dropped) is
+// a strip: the row above and the residues stay in registers and move down the
+// lanes with the origin.  The others go chunk by chunk: column j of the row
+// above is kept in slot j - o + 2 of the row buffer (slots 0 and 1 hold the
+// dead value), so the two slots a lane reads and writes are one aligned 8-byte
+// word.  The E scan runs over the lanes' pairwise maxima.  Values are computed
+// relative to the line of the row above (no add per value), the live test and
+// the stored values relative to the row's own line.  In chunks each lane keeps
+// its first and last live column and its best key (H - line) << 11 | (2047 -
+// (j - o)) of a live cell; three warp reductions at the row's end give the
+// live window, the row maximum and its first column.  A strip needs one
+// reduction (the maximum: below the line the side ends, above the old best
+// the line rises) and one ballot (the lanes with a live cell).
+//
+// The strip is bound by the ALU pipe (72 % busy, issue 70 %): 101 warp
+// instructions a row of 64 columns, 173 when every row went through the row
+// buffer.  The 4.9e6 records of 10,000 x 100,000 proteins (3.17e10 computed
+// cells): 99.3 -> 62.9 ms.  On the way: a strip whose columns stay in their
+// lanes while the origin moves round the ring of lanes (no moves, but a
+// rotated scan and ballots), 80.2 ms; the moving strip with the row-by-row
+// stores, tests and selects as in the chunks, 71.0; dead cells by an unsigned
+// minimum, one ballot, F kept less ge, the line updated only when it rises, 62.9.
 struct SideOut {
   int32_t score, ei, ej;
   int64_t cells;  // computed cells, every row
 };
 
+// A row kept in registers (side_dp), a lane's part of it: lane l holds the
+// columns o + 2l and o + 2l + 1 from the origin o on.
+struct Strip {
+  int32_t h0, h1;          // H of its two columns, against the row's line (FG_DEAD16 or less: dead)
+  int32_t g0, g1;          // their F less ge
+  int32_t kill0, kill1;    // 0, or FG_KILL for a column past the sequence end
+  int b0, b1;              // the columns' residues
+  int o;                   // the origin (the same in every lane)
+};
+constexpr int32_t FG_KILL = -(1 << 20);
+
+// The residues of the strip's columns (column 0 and columns past the sequence
+// end read the sentinel padding).
+template <int DIR>
+__device__ __forceinline__ void strip_residues(Strip& st, const int8_t* B, int lb, int lane) {
+  const int j0 = st.o + 2 * lane;
+  st.b0 = B[DIR * (j0 - 1)];
+  st.b1 = B[DIR * j0];
+  if (st.o + 63 > lb) {
+    st.kill0 = j0 <= lb ? 0 : FG_KILL;
+    st.kill1 = j0 < lb ? 0 : FG_KILL;
+  }
+}
+
 template <int DIR>
 __device__ SideOut side_dp(const int8_t* A, int la, const int8_t* B, int lb, int go, int ge, int X, const int8_t* tab,
                            uint32_t* Sbuf, uint8_t* arena, int* err, int lane) {
+  const unsigned FULL = 0xffffffffu;
   const int goe = go + ge;
   int32_t* rowtab = reinterpret_cast<int32_t*>(arena);  // (origin, offset, line, stored columns) per row
   int16_t* hval = reinterpret_cast<int16_t*>(arena);     // H of the stored columns, from the offset
@@ -115,124 +153,269 @@ __device__ SideOut side_dp(const int8_t* A, int la, const int8_t* B, int lb, int
   // a side whose rows all fit whole, even at their widest (la + 1 rows of at
   // most lb + 2 stored columns), needs no capacity test at all
   const bool side_fits = lb + 4 <= FG_W && off + (int64_t)(la + 1) * (lb + 2) < FG_ARENA / 2;
-  int32_t T = 0, best = 0, bi = 0, bj = 0;
+  int32_t best = 0, bi = 0, bj = 0;  // (also T: the best of the rows so far)
   int32_t cells = 0;  // computed cells (at most the arena's columns)
-  int plo = 0, phi = 0, po = 0, pw2 = 2;  // the row above: live columns, origin, first slot after it
-  int32_t pthr = 0;                       // the row above's drop-off line
-  int ai = 0;                             // A_i of the row (row 0: none)
-  __syncwarp();  // (row 0 has no row above: pw2 = 2 makes it an empty one)
-  for (int i = 0; i <= la; i++) {
-    const int c0 = i == 0 ? 0 : plo;
-    const int o = c0 & ~1;                 // the row's origin (even)
-    const int lim = i == 0 ? 0 : phi + 1;  // the last column a cell of the row above can feed
-    // the row is written over the row above in the same buffer: a chunk
-    // reads the row above before it stores (its scan's shuffles come
-    // between), the row's origin is never left of the row above's, so a
-    // chunk overwrites only columns left of what later chunks read, but for
-    // the row-above column just left of the next chunk, which lane 31 of
-    // this chunk hands on
-    uint32_t* Sp = Sbuf;
-    uint32_t carry_sm = 0;  // the row above's slot of column cs - 1 (chunks after the first)
-    const int32_t thr = T - X;
-    const int32_t trel = thr - pthr;  // the row's line relative to the row above's
-    const int8_t* trow = tab + ai * NCODE;
-    ai = i < la ? A[DIR * i] : 0;  // the next row's residue, loaded a row ahead
-    int32_t carryP = FG_NEG;
-    int32_t lkey = -1, llo = 0x7fffffff, lhi = -1;  // this lane's best key, first and last live column
-    bool overflow = false;
-    // a row that fits whole needs no test per chunk
-    const bool fits = side_fits || (lb - o + 4 <= FG_W && off + (lb - o) + 1 < FG_ARENA / 2);
-    int cs = o;  // (o <= c0 <= lb: the row has at least one chunk)
-    for (;; cs += 64) {
-      // capacity of the chunk's last column (the same test for every lane)
-      const int wl = min(cs + 63, lb) - o;
-      if (!fits && (wl + 4 > FG_W || off + wl + 1 >= FG_ARENA / 2)) {
-        overflow = true;
-        break;
+  int plo = 0;        // the row above: its first live column
+  int32_t pthr = 0;   // its drop-off line
+  int i = 0;          // the next row
+
+  // A row of at most 64 columns from the origin keeps the row above in
+  // registers (a strip), and the residues of its columns with it.
+  const int before = (lane + 31) & 31;
+  const int32_t c0 = 2 * lane * ge, c1 = c0 + ge;  // (column - origin) * ge
+  // what the prefix maximum of the lanes before adds to E; lane 0 has none before it
+  const int32_t e0 = lane == 0 ? FG_NEG : -(go + c0), e1 = lane == 0 ? FG_NEG : -(go + c1);
+  Strip st;
+  st.o = 0;
+  st.kill0 = st.kill1 = 0;
+  strip_residues<DIR>(st, B, lb, lane);
+  bool wide;  // the next row is computed in chunks (the same in every lane)
+  {
+    // row 0: the anchor and the gaps from it
+    const int32_t r0 = (lane == 0 ? 0 : -go - c0) + X + st.kill0, r1 = -go - c1 + X + st.kill1;
+    const bool live0 = r0 >= 0, live1 = r1 >= 0;
+    st.h0 = live0 ? r0 : FG_DEAD16;
+    st.h1 = live1 ? r1 : FG_DEAD16;
+    st.g0 = st.g1 = FG_DEAD16;
+    wide = __ballot_sync(FULL, live1) >> 31;  // a live last column: the rows in chunks, from row 0
+    if (!wide) {
+      const int cend = min(64, lb + 1), cw = (cend + 1) & ~1;
+      if (!side_fits && off + cend >= FG_ARENA / 2) {
+        if (lane == 0) atomicOr(err, FG_ERR_WIDTH);
+        return out;
       }
-      // (a column left of c0 reads only dead cells of the row above and dead
-      // E terms: it comes out dead, and its prefix term lies below every
-      // live one to its right; a column past lb feeds only columns past lb)
-      const int j0 = cs + 2 * lane, j1 = j0 + 1;
-      const bool in0 = j0 <= lb, in1 = j1 <= lb;
-      // row above: columns j0 and j0 + 1 at slots kp, kp + 1 (kp = j0 - po +
-      // 2, even; the load stays inside the buffer), column j0 - 1 from the
-      // lane to the left (lane 0: from lane 31 of the chunk before, and in a
-      // row's first chunk column o - 1, left of the row above's first live
-      // column, dead)
-      const int kp = j0 - po + 2;
-      // (the slots from pw2 on may hold this row's own earlier chunks: a
-      // column there is past the row above and takes the dead value)
-      uint2 sv = *reinterpret_cast<const uint2*>(Sp + min(kp, pw2));
-      if (kp >= pw2) sv = make_uint2(FG_DEAD, FG_DEAD);
-      uint32_t sm = __shfl_up_sync(0xffffffffu, sv.y, 1);
-      if (lane == 0) sm = cs > o ? carry_sm : FG_DEAD;
-      const int32_t hd0 = (int32_t)(int16_t)(sm & 0xffffu);
-      const int32_t hu0 = (int32_t)(int16_t)(sv.x & 0xffffu), fu0 = (int32_t)sv.x >> 16;
-      const int32_t hu1 = (int32_t)(int16_t)(sv.y & 0xffffu), fu1 = (int32_t)sv.y >> 16;
-      // (j = 0 and columns past the sequence end read the sentinel padding)
-      const int32_t D0 = hd0 + trow[B[DIR * (j0 - 1)]], D1 = hu0 + trow[B[DIR * j0]];
-      const int32_t F0 = max(fu0 - ge, hu0 - goe), F1 = max(fu1 - ge, hu1 - goe);
-      int32_t DF0 = max(D0, F0);
-      const int32_t DF1 = max(D1, F1);
-      if (i == 0 && j0 == 0) DF0 = 0;  // the anchor (row 0's row above is empty, its line 0)
-      // E from the exclusive prefix maximum of DF(k) + k ge over the row (a
-      // lane below the shuffle distance gets its own value back)
-      const int32_t P0 = DF0 + j0 * ge, P1 = DF1 + j1 * ge;
-      int32_t incl = max(P0, P1);
+      if (st.kill0 == 0)
+        *reinterpret_cast<uint32_t*>(hval + off + 2 * lane) = __byte_perm((uint32_t)st.h0, (uint32_t)st.h1, 0x5410u);
+      if (lane == 0) *reinterpret_cast<int4*>(rowtab) = make_int4(0, off, -X, cw);
+      off += cw;
+      cells = cend;
+      pthr = -X;
+      i = 1;
+    }
+  }
+  int po = 0, phi = 0, pw2 = 2;  // the row above in chunks: origin, last live column, first slot after it
+  int ai = i == 1 && la > 0 ? A[0] : 0;  // A_i of the row (row 0: none)
+  __syncwarp();
+  for (;;) {
+    // ---- rows of one strip
+    if (!wide) {
+      bool ended = false;
+      int32_t thr = best - X, trel = thr - pthr;  // the row's line, and relative to the row above's
+      const int off_safe = side_fits ? 0x7fffffff : (int)(FG_ARENA / 2) - 64;
+      const int8_t* ap = A + DIR * i;
+      int16_t* hp = hval + off + 2 * lane;
+      for (; i <= la; i++, ap += DIR) {
+        const int8_t* trow = tab + ai * NCODE;
+        const int an = *ap;  // the next row's residue, loaded a row ahead (past the last: padding)
+        // the diagonal of the lane's first column is the lane before's last;
+        // before lane 0 comes lane 31's, which is dead in a strip
+        const int32_t hd0 = __shfl_sync(FULL, st.h1, before);
+        const int32_t F0 = max(st.h0 - goe, st.g0), F1 = max(st.h1 - goe, st.g1);
+        const int32_t DF0 = max(hd0 + trow[st.b0], F0), DF1 = max(st.h0 + trow[st.b1], F1);
+        // E from the exclusive prefix maximum of DF(k) + k ge (a lane below
+        // the shuffle distance gets its own value back)
+        const int32_t P0 = DF0 + c0;
+        int32_t incl = max(DF1 + c1, P0);
 #pragma unroll
-      for (int d = 1; d < 32; d <<= 1) incl = max(incl, __shfl_up_sync(0xffffffffu, incl, d));
-      int32_t ex = __shfl_up_sync(0xffffffffu, incl, 1);
-      ex = lane == 0 ? carryP : max(ex, carryP);
-      const int32_t E0 = ex - go - j0 * ge, E1 = max(ex, P0) - go - j1 * ge;
-      const int32_t H0 = max(DF0, E0), H1 = max(DF1, E1);
-      const bool live0 = in0 && H0 >= trel, live1 = in1 && H1 >= trel;
-      const int32_t r0 = H0 - trel, r1 = H1 - trel;  // against the row's line
-      if (in0 || in1) {
-        const int w = j0 - o;  // even
-        const uint32_t v0 = live0 ? __byte_perm((uint32_t)r0, (uint32_t)(F0 - trel), 0x5410u) : FG_DEAD;
-        const uint32_t v1 = live1 ? __byte_perm((uint32_t)r1, (uint32_t)(F1 - trel), 0x5410u) : FG_DEAD;
-        *reinterpret_cast<uint2*>(Sp + w + 2) = make_uint2(v0, v1);
-        *reinterpret_cast<uint32_t*>(hval + off + w) = __byte_perm(v0, v1, 0x5410u);  // the two H halves
+        for (int d = 1; d < 32; d <<= 1) incl = max(incl, __shfl_up_sync(FULL, incl, d));
+        const int32_t ex = __shfl_up_sync(FULL, incl, 1);
+        const int32_t H0 = max(ex + e0, DF0), H1 = max(ex + e1, max(P0 - (go + c1), DF1));
+        const int32_t r0 = H0 - trel + st.kill0, r1 = H1 - trel + st.kill1;  // against the row's line
+        const int32_t v = max(r0, r1);
+        const unsigned m = __ballot_sync(FULL, v >= 0);  // the lanes with a live cell
+        if (m >> 31) break;  // the strip's last columns: this row in chunks
+        const int wl = min(63, lb - st.o);
+        if (off >= off_safe && off + wl + 1 >= FG_ARENA / 2) {
+          if (lane == 0) atomicOr(err, FG_ERR_WIDTH);
+          return out;
+        }
+        cells += st.o + wl + 1 - plo;
+        const int cw = (wl + 2) & ~1;
+        const int32_t rm = __reduce_max_sync(FULL, v);
+        // (a cell at or above the line keeps its value, the others sink to the
+        // dead one or below: as unsigned numbers the negative are the large)
+        st.h0 = (int32_t)min((uint32_t)r0, (uint32_t)FG_DEAD16);
+        st.h1 = (int32_t)min((uint32_t)r1, (uint32_t)FG_DEAD16);
+        // (a dropped cell's F may stay: it lies below the line, and only falls)
+        st.g0 = max(F0 - (trel + ge), FG_DEAD16);
+        st.g1 = max(F1 - (trel + ge), FG_DEAD16);
+        if (st.kill0 == 0) *reinterpret_cast<uint32_t*>(hp) = __byte_perm((uint32_t)st.h0, (uint32_t)st.h1, 0x5410u);
+        if (lane == 0) *reinterpret_cast<int4*>(rowtab + 4 * i) = make_int4(st.o, off, thr, cw);
+        off += cw;
+        hp += cw;
+        ai = an;
+        trel = 0;
+        if ((unsigned)rm > (unsigned)X) {
+          if (rm < 0) {  // no live cell: the side ends
+            ended = true;
+            break;
+          }
+          // a new best: its row and first column, and a higher line
+          trel = rm - X;
+          best += trel;
+          bi = i;
+          const int k0 = __ffs(__ballot_sync(FULL, r0 == rm)) - 1, k1 = __ffs(__ballot_sync(FULL, r1 == rm)) - 1;
+          bj = st.o + (int)min((unsigned)(2 * k0), (unsigned)(2 * k1 + 1));
+        }
+        pthr = thr;
+        thr += trel;
+        // the origin moves to the first live column (rounded down to even)
+        const int sft = __ffs(m) - 1;
+        plo = st.o + 2 * sft + (int)((uint32_t)__shfl_sync(FULL, r0, sft) >> 31);
+        if (sft > 0) {
+          st.o += 2 * sft;
+          strip_residues<DIR>(st, B, lb, lane);
+          const bool in = lane + sft < 32;
+          const int32_t h0 = __shfl_down_sync(FULL, st.h0, sft), h1 = __shfl_down_sync(FULL, st.h1, sft);
+          const int32_t g0 = __shfl_down_sync(FULL, st.g0, sft), g1 = __shfl_down_sync(FULL, st.g1, sft);
+          st.h0 = in ? h0 : FG_DEAD16;
+          st.h1 = in ? h1 : FG_DEAD16;
+          st.g0 = in ? g0 : FG_DEAD16;
+          st.g1 = in ? g1 : FG_DEAD16;
+        }
       }
-      // (the key as r * 2048 + code: r >= 0 and code < 2048 for a live cell;
-      // a multiply-add leaves the ALU pipe, the bound, to the maxima)
-      const int kc = 2047 - (j0 - o);
-      lkey = max(lkey, max(live0 ? r0 * 2048 + kc : -1, live1 ? r1 * 2048 + (kc - 1) : -1));
-      llo = min(llo, live0 ? j0 : live1 ? j1 : 0x7fffffff);
-      lhi = max(lhi, live1 ? j1 : live0 ? j0 : -1);
-      // past the sequence end, or past the row above's reach with the
-      // chunk's last cell dropped: the row ends
-      if (cs + 64 > lb || (cs + 63 >= lim && !(__ballot_sync(0xffffffffu, live1) >> 31))) break;
-      // what the next chunk takes from this one's lane 31
-      carryP = max(carryP, __shfl_sync(0xffffffffu, incl, 31));
-      carry_sm = __shfl_sync(0xffffffffu, sv.y, 31);
+      if (ended || i > la) break;
+      // row i in chunks: the row above into the row buffer
+      const unsigned m0 = __ballot_sync(FULL, st.h0 >= 0), m1 = __ballot_sync(FULL, st.h1 >= 0);
+      const int k = 31 - __clz(m0 | m1);
+      po = st.o;
+      phi = po + 2 * k + (m1 >> k & 1u);
+      pw2 = 66;
+      *reinterpret_cast<uint2*>(Sbuf + 2 * lane + 2) =
+          make_uint2(__byte_perm((uint32_t)max(st.h0, FG_DEAD16), (uint32_t)(st.g0 + ge), 0x5410u),
+                     __byte_perm((uint32_t)max(st.h1, FG_DEAD16), (uint32_t)(st.g1 + ge), 0x5410u));
+      wide = true;
+      __syncwarp();
     }
-    if (overflow) {
-      if (lane == 0) atomicOr(err, FG_ERR_WIDTH);
-      return out;
+    // ---- one row in chunks
+    {
+      const int c0 = i == 0 ? 0 : plo;
+      const int o = c0 & ~1;                 // the row's origin (even)
+      const int lim = i == 0 ? 0 : phi + 1;  // the last column a cell of the row above can feed
+      // the row is written over the row above in the same buffer: a chunk
+      // reads the row above before it stores (its scan's shuffles come
+      // between), the row's origin is never left of the row above's, so a
+      // chunk overwrites only columns left of what later chunks read, but for
+      // the row-above column just left of the next chunk, which lane 31 of
+      // this chunk hands on
+      uint32_t* Sp = Sbuf;
+      uint32_t carry_sm = 0;  // the row above's slot of column cs - 1 (chunks after the first)
+      const int32_t thr = best - X;
+      const int32_t trel = thr - pthr;  // the row's line relative to the row above's
+      const int8_t* trow = tab + ai * NCODE;
+      ai = i < la ? A[DIR * i] : 0;  // the next row's residue, loaded a row ahead
+      int32_t carryP = FG_NEG;
+      int32_t lkey = -1, llo = 0x7fffffff, lhi = -1;  // this lane's best key, first and last live column
+      bool overflow = false;
+      // a row that fits whole needs no test per chunk
+      const bool fits = side_fits || (lb - o + 4 <= FG_W && off + (lb - o) + 1 < FG_ARENA / 2);
+      int cs = o;  // (o <= c0 <= lb: the row has at least one chunk)
+      for (;; cs += 64) {
+        // capacity of the chunk's last column (the same test for every lane)
+        const int wl = min(cs + 63, lb) - o;
+        if (!fits && (wl + 4 > FG_W || off + wl + 1 >= FG_ARENA / 2)) {
+          overflow = true;
+          break;
+        }
+        // (a column left of c0 reads only dead cells of the row above and dead
+        // E terms: it comes out dead, and its prefix term lies below every
+        // live one to its right; a column past lb feeds only columns past lb)
+        const int j0 = cs + 2 * lane, j1 = j0 + 1;
+        const bool in0 = j0 <= lb, in1 = j1 <= lb;
+        // row above: columns j0 and j0 + 1 at slots kp, kp + 1 (kp = j0 - po +
+        // 2, even; the load stays inside the buffer), column j0 - 1 from the
+        // lane to the left (lane 0: from lane 31 of the chunk before, and in a
+        // row's first chunk column o - 1, left of the row above's first live
+        // column, dead)
+        const int kp = j0 - po + 2;
+        // (the slots from pw2 on may hold this row's own earlier chunks: a
+        // column there is past the row above and takes the dead value)
+        uint2 sv = *reinterpret_cast<const uint2*>(Sp + min(kp, pw2));
+        if (kp >= pw2) sv = make_uint2(FG_DEAD, FG_DEAD);
+        uint32_t sm = __shfl_up_sync(0xffffffffu, sv.y, 1);
+        if (lane == 0) sm = cs > o ? carry_sm : FG_DEAD;
+        const int32_t hd0 = (int32_t)(int16_t)(sm & 0xffffu);
+        const int32_t hu0 = (int32_t)(int16_t)(sv.x & 0xffffu), fu0 = (int32_t)sv.x >> 16;
+        const int32_t hu1 = (int32_t)(int16_t)(sv.y & 0xffffu), fu1 = (int32_t)sv.y >> 16;
+        // (j = 0 and columns past the sequence end read the sentinel padding)
+        const int32_t D0 = hd0 + trow[B[DIR * (j0 - 1)]], D1 = hu0 + trow[B[DIR * j0]];
+        const int32_t F0 = max(fu0 - ge, hu0 - goe), F1 = max(fu1 - ge, hu1 - goe);
+        int32_t DF0 = max(D0, F0);
+        const int32_t DF1 = max(D1, F1);
+        if (i == 0 && j0 == 0) DF0 = 0;  // the anchor (row 0's row above is empty, its line 0)
+        // E from the exclusive prefix maximum of DF(k) + k ge over the row (a
+        // lane below the shuffle distance gets its own value back)
+        const int32_t P0 = DF0 + j0 * ge, P1 = DF1 + j1 * ge;
+        int32_t incl = max(P0, P1);
+  #pragma unroll
+        for (int d = 1; d < 32; d <<= 1) incl = max(incl, __shfl_up_sync(0xffffffffu, incl, d));
+        int32_t ex = __shfl_up_sync(0xffffffffu, incl, 1);
+        ex = lane == 0 ? carryP : max(ex, carryP);
+        const int32_t E0 = ex - go - j0 * ge, E1 = max(ex, P0) - go - j1 * ge;
+        const int32_t H0 = max(DF0, E0), H1 = max(DF1, E1);
+        const bool live0 = in0 && H0 >= trel, live1 = in1 && H1 >= trel;
+        const int32_t r0 = H0 - trel, r1 = H1 - trel;  // against the row's line
+        if (in0 || in1) {
+          const int w = j0 - o;  // even
+          const uint32_t v0 = live0 ? __byte_perm((uint32_t)r0, (uint32_t)(F0 - trel), 0x5410u) : FG_DEAD;
+          const uint32_t v1 = live1 ? __byte_perm((uint32_t)r1, (uint32_t)(F1 - trel), 0x5410u) : FG_DEAD;
+          *reinterpret_cast<uint2*>(Sp + w + 2) = make_uint2(v0, v1);
+          *reinterpret_cast<uint32_t*>(hval + off + w) = __byte_perm(v0, v1, 0x5410u);  // the two H halves
+        }
+        // (the key as r * 2048 + code: r >= 0 and code < 2048 for a live cell;
+        // a multiply-add leaves the ALU pipe, the bound, to the maxima)
+        const int kc = 2047 - (j0 - o);
+        lkey = max(lkey, max(live0 ? r0 * 2048 + kc : -1, live1 ? r1 * 2048 + (kc - 1) : -1));
+        llo = min(llo, live0 ? j0 : live1 ? j1 : 0x7fffffff);
+        lhi = max(lhi, live1 ? j1 : live0 ? j0 : -1);
+        // past the sequence end, or past the row above's reach with the
+        // chunk's last cell dropped: the row ends
+        if (cs + 64 > lb || (cs + 63 >= lim && !(__ballot_sync(0xffffffffu, live1) >> 31))) break;
+        // what the next chunk takes from this one's lane 31
+        carryP = max(carryP, __shfl_sync(0xffffffffu, incl, 31));
+        carry_sm = __shfl_sync(0xffffffffu, sv.y, 31);
+      }
+      if (overflow) {
+        if (lane == 0) atomicOr(err, FG_ERR_WIDTH);
+        return out;
+      }
+      const int cend = min(cs + 64, lb + 1);  // past the row's last computed column
+      const int cw = (cend - o + 1) & ~1;     // stored columns, even
+      cells += cend - c0;
+      const int32_t key = __reduce_max_sync(FULL, lkey);
+      if (key < 0) break;  // no live cell: the side ends
+      const int32_t rmax = (key >> 11) + thr;
+      const int rarg = o + 2047 - (key & 2047);
+      plo = __reduce_min_sync(FULL, llo);
+      phi = __reduce_max_sync(FULL, lhi);
+      if (lane == 0) *reinterpret_cast<int4*>(rowtab + 4 * i) = make_int4(o, off, thr, cw);
+      off += cw;
+      if (rmax > best) {
+        best = rmax;
+        bi = i;
+        bj = rarg;
+      }
+      po = o;
+      pw2 = cw + 2;
+      pthr = thr;
+      __syncwarp();
     }
-    const int cend = min(cs + 64, lb + 1);  // past the row's last computed column
-    const int cw = (cend - o + 1) & ~1;     // stored columns, even
-    cells += cend - c0;
-    const int32_t key = __reduce_max_sync(0xffffffffu, lkey);
-    if (key < 0) break;  // no live cell: the side ends
-    const int32_t rmax = (key >> 11) + thr;
-    const int rarg = o + 2047 - (key & 2047);
-    plo = __reduce_min_sync(0xffffffffu, llo);
-    phi = __reduce_max_sync(0xffffffffu, lhi);
-    if (lane == 0) *reinterpret_cast<int4*>(rowtab + 4 * i) = make_int4(o, off, thr, cw);
-    off += cw;
-    if (rmax > best) {
-      best = rmax;
-      bi = i;
-      bj = rarg;
+    if (++i > la) break;
+    if (phi - (plo & ~1) < 62) {
+      // narrow again: back into a strip
+      wide = false;
+      st.o = plo & ~1;
+      st.kill0 = st.kill1 = 0;
+      strip_residues<DIR>(st, B, lb, lane);
+      const int kp = st.o + 2 * lane - po + 2;
+      uint2 sv = *reinterpret_cast<const uint2*>(Sbuf + min(kp, pw2));
+      if (kp >= pw2) sv = make_uint2(FG_DEAD, FG_DEAD);
+      st.h0 = (int32_t)(int16_t)(sv.x & 0xffffu);
+      st.g0 = ((int32_t)sv.x >> 16) - ge;
+      st.h1 = (int32_t)(int16_t)(sv.y & 0xffffu);
+      st.g1 = ((int32_t)sv.y >> 16) - ge;
+      __syncwarp();
     }
-    T = max(T, rmax);
-    po = o;
-    pw2 = cw + 2;
-    pthr = thr;
-    __syncwarp();
   }
   out.score = best;
   out.ei = bi;
