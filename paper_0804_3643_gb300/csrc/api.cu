@@ -778,41 +778,40 @@ int plast_index_bank(const int8_t* codes, const int64_t* seq_off, int32_t n_seqs
                                  cudaMemcpyDeviceToDevice, st))))
       return fail(rc);
     if ((rc = ck(launch_build_pad(codes, d_seq_off, n_seqs, n_res, 20, b->pad, d_bad, st)))) return fail(rc);
-    const int64_t ix_tile = index_tile(n_pad), n_tiles = (n_pad + ix_tile - 1) / ix_tile;
-    const int64_t n_cells = (int64_t)NKEYS * n_tiles;
+    const IndexShape shape = index_shape(n_pad);
+    const int64_t n_cells = index_cells(shape);
     int32_t* d_hist;
     int64_t *d_off, *d_total;
     if ((rc = ck(sc.get(&d_hist, n_cells)))) return fail(rc);
     if ((rc = ck(sc.get(&d_off, n_cells)))) return fail(rc);
     if ((rc = ck(sc.get(&d_total, 1)))) return fail(rc);
-    if ((rc = ck(launch_index_hist(b->pad, n_pad, ix_tile, n_tiles, d_hist, st)))) return fail(rc);
+    if ((rc = ck(launch_index_hist(b->pad, n_pad, shape, d_hist, st)))) return fail(rc);
     void* stmp;
     size_t stb = scan_tmp_bytes(n_cells);
     if ((rc = ck(sc.get((char**)&stmp, stb)))) return fail(rc);
     if ((rc = ck(scan_exclusive(d_hist, d_off, n_cells, d_total, stmp, stb, st)))) return fail(rc);
-    int64_t n_idx = 0;
+    if ((rc = ck(launch_index_key_off(d_off, shape, b->key_off, st)))) return fail(rc);
+    uint32_t* by_pos;
+    uint8_t* by_lo;
+    const size_t room = (size_t)std::max<int64_t>(n_res, 1);  // a word per residue at most
+    if ((rc = ck(sc.get(&by_pos, room)))) return fail(rc);
+    if ((rc = ck(sc.get(&by_lo, room)))) return fail(rc);
+    if ((rc = ck(launch_index_split(b->pad, n_pad, shape, d_off, by_pos, by_lo, st)))) return fail(rc);
     int h_bad = 0;
-    if ((rc = ck(cudaMemcpyAsync(&n_idx, d_total, sizeof(int64_t), cudaMemcpyDeviceToHost, st)))) return fail(rc);
-    if ((rc = ck(cudaMemcpyAsync(&h_bad, d_bad, sizeof(int), cudaMemcpyDeviceToHost, st)))) return fail(rc);
-    if ((rc = ck(cudaStreamSynchronize(st)))) return fail(rc);
-    if (h_bad) return fail(PLAST_E_INVALID);
-    b->n_idx = n_idx;
-    if ((rc = ck(dev_alloc_async((void**)&b->pos, (size_t)std::max<int64_t>(n_idx, 1) * sizeof(uint32_t), st))))
-      return fail(rc);
-    int64_t* d_offT;
-    if ((rc = ck(sc.get(&d_offT, n_cells)))) return fail(rc);
-    if ((rc = ck(launch_index_finish(b->pad, n_pad, ix_tile, n_tiles, d_off, d_offT, d_total, b->key_off, b->pos,
-                                     st))))
-      return fail(rc);
     b->h_key_off.resize(NKEYS + 1);
     if ((rc = ck(cudaMemcpyAsync(b->h_key_off.data(), b->key_off, (NKEYS + 1) * sizeof(int64_t),
                                  cudaMemcpyDeviceToHost, st))))
       return fail(rc);
+    if ((rc = ck(cudaMemcpyAsync(&h_bad, d_bad, sizeof(int), cudaMemcpyDeviceToHost, st)))) return fail(rc);
     if ((rc = ck(cudaStreamSynchronize(st)))) return fail(rc);
-    // the windows are laid out while the caller goes on (later calls wait on
+    if (h_bad) return fail(PLAST_E_INVALID);
+    const int64_t n_idx = b->n_idx = b->h_key_off[NKEYS];
+    if ((rc = ck(dev_alloc_async((void**)&b->pos, (size_t)std::max<int64_t>(n_idx, 1) * sizeof(uint32_t), st))))
+      return fail(rc);
+    // the lists are laid out while the caller goes on (later calls wait on
     // b->ready)
     if ((rc = ck(dev_alloc_async((void**)&b->nb, (size_t)std::max<int64_t>(n_idx, 1) * WIN, st)))) return fail(rc);
-    if ((rc = ck(launch_neighbourhoods(b->pad, b->pos, n_idx, b->nb, st)))) return fail(rc);
+    if ((rc = ck(launch_index_fill(b->pad, shape, d_off, by_pos, by_lo, b->pos, b->nb, st)))) return fail(rc);
     if ((rc = ck(cudaEventCreateWithFlags(&b->ready, cudaEventDisableTiming)))) return fail(rc);
     if ((rc = ck(cudaEventRecord(b->ready, st)))) return fail(rc);
   }

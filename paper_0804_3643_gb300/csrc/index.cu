@@ -74,19 +74,37 @@ __global__ void k_build_pad(const int8_t* codes, const int64_t* seq_off, int32_t
   if (b) atomicOr(bad, 1);
 }
 
-// Stage 0's lookup table and lists (Section 3.3.1) as a stable counting
-// sort of the padded positions by key.  A word is indexed when its four
-// letters are residues (codes below 20: no stop, no sentinel, so no word
-// crosses a sequence end).  The padded bank is cut into tiles of T positions
-// (a multiple of 4096, chosen so that the tiles keep the GPU busy); pass 1
-// counts each tile's words per key, an exclusive scan of the counts in
-// key-major order gives every (key, tile) its first slot (and, at (k, 0), the
-// CSR offset of key k), pass 2 walks each tile in position order with one
-// warp and writes each word's position into its key's slots, so positions
-// increase within a key.
-constexpr int IX_THREADS = 256;
+// Stage 0's lookup table and lists (Section 3.3.1) as a stable counting sort
+// of the padded positions by key, high digit first.  A word is indexed when
+// its four letters are residues (codes below 20: no stop, no sentinel, so no
+// word crosses a sequence end).  The key's high digit (key / 128) names its
+// bucket, of 69.  The padded bank is cut into chunks of 8192 positions and
+// these into groups (IndexShape):
+//   k_index_hist   counts each chunk's words per bucket and each group's per
+//                  key; an exclusive scan of the two tables, bucket-major and
+//                  key-major, gives every (bucket, chunk) and every (key,
+//                  group) its first slot, and with it the CSR offsets;
+//   k_index_split  sorts each chunk by bucket in shared memory: positions and
+//                  low digits move to their buckets, in position order;
+//   k_index_fill   takes a bucket's words of one group, sorts them by the low
+//                  digit and writes each key's run of positions and windows.
+// Why two digits: with 8,800 destinations at once a word's 4-byte position and
+// 48-byte window go to places that no other word of the same few microseconds
+// touches, and every store is a partial line.  Split first, the runs are some
+// 90 words (split) and 47 words (fill) long, and the words a CTA of k_index_fill
+// holds come from a stretch of 1 MB or so of the bank, in L2 for all buckets.
+// For 166 M words in 206 M padded positions: hist 0.43 ms, split 0.98, fill
+// 2.96; one scatter over all keys took 3.69 and the windows, gathered in key
+// order over the whole bank, 4.09 (sorting both digits of a chunk in one CTA
+// and storing the windows from there: 8.5).
+constexpr int IX_THREADS = 512;
+constexpr int IX_WARPS = IX_THREADS / 32;
 constexpr int IX_PER = 16;                      // positions per thread and chunk
-constexpr int IX_CHUNK = IX_THREADS * IX_PER;   // 4096
+constexpr int IX_CHUNK = IX_THREADS * IX_PER;   // 8192
+constexpr int IX_LO = 128;                      // keys per bucket
+constexpr int IX_LO_BITS = 7;
+constexpr int IX_BUCKETS = (NKEYS + IX_LO - 1) / IX_LO;
+static_assert(1 << IX_LO_BITS == IX_LO, "the low digit");
 
 // Keys of the 16 words at p0 .. p0 + 15 from five aligned words of pad (p0 is
 // a multiple of 16; a thread at or past n_pad reads nothing, the others at
@@ -141,165 +159,306 @@ __device__ __forceinline__ void load_classes(int8_t* cls2, int8_t* cls3) {
   }
 }
 
-// Pass 1: hist[k * n_tiles + t] = words of key k in tile t.
-__global__ void __launch_bounds__(IX_THREADS) k_index_hist(const int8_t* pad, int64_t n_pad, int64_t tile,
-                                                           int64_t n_tiles, int32_t* hist) {
+// hist[b * n_chunks + c] = words of bucket b in chunk c; behind those,
+// hist_key[k * n_groups + g] += words of key k in the CTA's chunks, `per`
+// consecutive ones of group g (several CTAs a group: added up in memory).
+__global__ void __launch_bounds__(IX_THREADS) k_index_hist(const int8_t* pad, int64_t n_pad, IndexShape sh,
+                                                           int32_t* hist) {
   __shared__ int32_t cnt[NKEYS];
+  __shared__ int32_t bucket[IX_BUCKETS];
   __shared__ int8_t cls2[NAA], cls3[NAA];
   for (int k = threadIdx.x; k < NKEYS; k += IX_THREADS) cnt[k] = 0;
+  if (threadIdx.x < IX_BUCKETS) bucket[threadIdx.x] = 0;
   load_classes(cls2, cls3);
   __syncthreads();
-  const int64_t base = (int64_t)blockIdx.x * tile;
-  for (int64_t c = 0; c < tile; c += IX_CHUNK) {
+  const int64_t c0 = (int64_t)blockIdx.x * sh.per, c1 = min(c0 + sh.per, sh.n_chunks);
+  for (int64_t c = c0; c < c1; c++) {
     int32_t key[IX_PER];
-    const uint32_t valid = word_keys16(pad, base + c + (int64_t)threadIdx.x * IX_PER, n_pad, cls2, cls3, key);
+    const uint32_t valid = word_keys16(pad, c * IX_CHUNK + threadIdx.x * IX_PER, n_pad, cls2, cls3, key);
 #pragma unroll
     for (int j = 0; j < IX_PER; j++)
-      if (valid >> j & 1) atomicAdd(&cnt[key[j]], 1);
+      if (valid >> j & 1) {
+        atomicAdd(&cnt[key[j]], 1);
+        atomicAdd(&bucket[key[j] >> IX_LO_BITS], 1);
+      }
+    __syncthreads();
+    if (threadIdx.x < IX_BUCKETS) {
+      hist[threadIdx.x * sh.n_chunks + c] = bucket[threadIdx.x];
+      bucket[threadIdx.x] = 0;
+    }
+    __syncthreads();
   }
-  __syncthreads();
-  for (int k = threadIdx.x; k < NKEYS; k += IX_THREADS) hist[(int64_t)k * n_tiles + blockIdx.x] = cnt[k];
+  int32_t* hist_key = hist + IX_BUCKETS * sh.n_chunks + c0 / sh.group;
+  for (int k = threadIdx.x; k < NKEYS; k += IX_THREADS)
+    if (cnt[k]) atomicAdd(&hist_key[k * sh.n_groups], cnt[k]);
 }
 
-// offT[t * NKEYS + k] = off[k * n_tiles + t]: the scanned slots tile-major,
-// so that each tile of pass 2 reads its keys' slots contiguously (32 x 32
-// blocks through shared memory, reads and writes coalesced).
-__global__ void k_index_transpose(const int64_t* off, int64_t n_tiles, int64_t* offT) {
-  __shared__ int64_t blk[32][33];
-  const int64_t k0 = (int64_t)blockIdx.y * 32, t0 = (int64_t)blockIdx.x * 32;
-  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-    const int64_t k = k0 + r, t = t0 + threadIdx.x;
-    if (k < NKEYS && t < n_tiles) blk[r][threadIdx.x] = off[k * n_tiles + t];
-  }
-  __syncthreads();
-  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-    const int64_t t = t0 + r, k = k0 + threadIdx.x;
-    if (k < NKEYS && t < n_tiles) offT[t * NKEYS + k] = blk[threadIdx.x][r];
-  }
-}
-
-// key_off[k] = first slot of key k (its tile-0 slot), key_off[NKEYS] = total.
-__global__ void k_index_key_off(const int64_t* off, int64_t n_tiles, const int64_t* total, int64_t* key_off) {
+// key_off[k] = first slot of key k (off: the scanned tables; the key table's
+// slots start after the bucket table's total, which is the number of words).
+__global__ void k_index_key_off(const int64_t* off, IndexShape sh, int64_t* key_off) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < NKEYS) key_off[k] = off[(int64_t)k * n_tiles];
-  if (k == NKEYS) key_off[k] = *total;
+  const int64_t* off_key = off + IX_BUCKETS * sh.n_chunks;
+  if (k < NKEYS) key_off[k] = off_key[k * sh.n_groups] - off_key[0];
+  if (k == NKEYS) key_off[k] = off_key[0];
 }
 
-// Pass 2: one warp per tile, in blocks of 512 positions: each lane computes
-// the keys of 16 consecutive positions from one 16-byte load (the next
-// block's load in flight meanwhile) and parks them in shared memory; the
-// block is then ranked 32 positions at a time in position order, lanes
-// holding the same key taking consecutive slots in lane order.  The 16 match
-// masks of a block are formed before the slots are taken, so only the
-// per-key slot counter orders the steps.  (The scattered 4-byte position
-// stores bound this kernel: more, smaller tiles shorten each key's run of
-// slots per tile and make it slower, not faster.)
-constexpr int IX_BLOCK = 32 * IX_PER;  // 512 positions
-__global__ void __launch_bounds__(32) k_index_scatter(const int8_t* pad, int64_t n_pad, int64_t tile,
-                                                      const int64_t* offT, uint32_t* pos) {
-  __shared__ int32_t next[NKEYS];
-  __shared__ int16_t kb[IX_BLOCK];
-  __shared__ int8_t cls2[NAA], cls3[NAA];
-  const int lane = threadIdx.x;
-  const int64_t* my_off = offT + (int64_t)blockIdx.x * NKEYS;
-#pragma unroll 8
-  for (int k = lane; k < NKEYS; k += 32) next[k] = (int32_t)my_off[k];
-  load_classes(cls2, cls3);
-  __syncwarp();
-  const int64_t base = (int64_t)blockIdx.x * tile, end = min(base + tile, n_pad);
-  uint32_t w[5];
-  load20(pad, base + (int64_t)lane * IX_PER, n_pad, w);
-  for (int64_t q0 = base; q0 < end; q0 += IX_BLOCK) {
-    {
-      uint32_t wn[5];
-      load20(pad, q0 + IX_BLOCK < end ? q0 + IX_BLOCK + (int64_t)lane * IX_PER : n_pad, n_pad, wn);
-      const int64_t p0 = q0 + (int64_t)lane * IX_PER;
-      int32_t key[IX_PER];
-      const uint32_t valid = keys16_from(w, cls2, cls3, key);
+// Four bytes from any offset of a 4-byte aligned array.
+__device__ __forceinline__ uint32_t word_at(const uint8_t* bytes, int at) {
+  const uint32_t* w = reinterpret_cast<const uint32_t*>(bytes + (at & ~3));
+  return __funnelshift_r(w[0], w[1], 8 * (at & 3));
+}
+
+// Counters of a stable counting pass over up to 128 digits: one column per
+// warp, the columns WARPS + 2 apart so that a warp's digits spread over the
+// banks.
+template <int WARPS>
+struct RankSmem {
+  static constexpr int COL = WARPS + 2;
+  uint16_t cnt[IX_LO * COL];
+  int32_t wsum[WARPS];
+
+  __device__ void clear() {
+    for (int k = threadIdx.x; k < IX_LO * COL / 2; k += 32 * WARPS) reinterpret_cast<uint32_t*>(cnt)[k] = 0;
+  }
+  // Rank of this lane's word among those of its digit that its warp has met.
+  // (Seven ballots find the lanes of the same digit faster than one
+  // match.any: the pass over 205 M positions 0.98 ms against 1.23.)
+  __device__ int rank(int warp, int lane, int digit, bool ok) {
+    unsigned peers = __ballot_sync(0xffffffffu, ok);
 #pragma unroll
-      for (int j = 0; j < IX_PER; j++)
-        kb[lane * IX_PER + j] = (int16_t)((valid >> j & 1) && p0 + j < end ? key[j] : -1);
-#pragma unroll
-      for (int c = 0; c < 5; c++) w[c] = wn[c];
+    for (int k = 0; k < IX_LO_BITS; k++) {
+      const bool bit = digit >> k & 1;
+      const unsigned m = __ballot_sync(0xffffffffu, bit);
+      peers &= bit ? m : ~m;
     }
+    uint16_t* c = cnt + digit * COL + warp;
+    const int have = ok ? *c : 0;
     __syncwarp();
-    int k[IX_PER];
-    unsigned peers[IX_PER];
-#pragma unroll
-    for (int j = 0; j < IX_PER; j++) {
-      k[j] = kb[32 * j + lane];
-      peers[j] = __match_any_sync(0xffffffffu, k[j] >= 0 ? k[j] : NKEYS + lane);
-    }
-#pragma unroll
-    for (int j = 0; j < IX_PER; j++) {
-      const int leader = __ffs(peers[j]) - 1;
-      int slot = 0;
-      if (k[j] >= 0 && lane == leader) {
-        slot = next[k[j]];
-        next[k[j]] = slot + __popc(peers[j]);
-      }
-      slot = __shfl_sync(0xffffffffu, slot, leader) + __popc(peers[j] & ((1u << lane) - 1u));
-      if (k[j] >= 0) pos[slot] = (uint32_t)(q0 + 32 * j + lane);
-    }
+    if (ok && lane == __ffs(peers) - 1) *c = (uint16_t)(have + __popc(peers));
     __syncwarp();
+    return have + __popc(peers & ((1u << lane) - 1u));
+  }
+  // Counts to first places, digit by digit, the warps in order within one;
+  // the total.  Between barriers of its own.
+  __device__ int scan() {
+    constexpr int PER = IX_LO * WARPS / (32 * WARPS);  // 4 counters a thread
+    constexpr int PER_DIGIT = WARPS / PER;             // threads a digit
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    __syncthreads();
+    uint16_t* c = cnt + (t / PER_DIGIT) * COL + (t % PER_DIGIT) * PER;
+    const int c0 = c[0], c1 = c[1], c2 = c[2], c3 = c[3];
+    int x = c0 + c1 + c2 + c3;
+    const int mine = x;
+#pragma unroll
+    for (int d = 1; d < 32; d *= 2) {
+      const int y = __shfl_up_sync(0xffffffffu, x, d);
+      if (lane >= d) x += y;
+    }
+    if (lane == 31) wsum[warp] = x;
+    __syncthreads();
+    int before = 0, total = 0;
+#pragma unroll
+    for (int w = 0; w < WARPS; w++) {
+      const int v = wsum[w];
+      if (w < warp) before += v;
+      total += v;
+    }
+    const int e = before + x - mine;
+    c[0] = (uint16_t)e;
+    c[1] = (uint16_t)(e + c0);
+    c[2] = (uint16_t)(e + c0 + c1);
+    c[3] = (uint16_t)(e + c0 + c1 + c2);
+    __syncthreads();
+    return total;
+  }
+  __device__ int place(int warp, int digit, int rank) const { return cnt[digit * COL + warp] + rank; }
+};
+
+struct SplitSmem {
+  uint32_t el[IX_CHUNK];                        // key << 14 | offset in the chunk, by bucket
+  alignas(16) uint8_t code[IX_CHUNK + 16];
+  int32_t slot[IX_BUCKETS];                     // first slot of each bucket less the index of its first word
+  RankSmem<IX_WARPS> rank;
+  int8_t cls2[NAA], cls3[NAA];
+};
+static_assert(IX_CHUNK <= 1 << 14 && NKEYS <= 1 << 14, "packing");
+static_assert(sizeof(SplitSmem) <= 48 * 1024, "static shared memory");
+
+// Waits on shared memory, one chunk a CTA and three CTAs an SM (four: 1.00 ms
+// for 0.98 at 206 M positions, their 32 registers spill).
+__global__ void __launch_bounds__(IX_THREADS, 3) k_index_split(const int8_t* pad, int64_t n_pad, IndexShape sh,
+                                                               const int64_t* off, uint32_t* by_pos,
+                                                               uint8_t* by_lo) {
+  __shared__ SplitSmem sm;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int64_t c = blockIdx.x, q0 = c * IX_CHUNK;
+  const uint4 gap = make_uint4(0x01010101u * SENTINEL, 0x01010101u * SENTINEL, 0x01010101u * SENTINEL,
+                               0x01010101u * SENTINEL);
+  // from n_pad on the words hold a sentinel; the bank's trailing slack covers the reads
+  const int64_t p = q0 + 16 * t;
+  *reinterpret_cast<uint4*>(sm.code + 16 * t) = p < n_pad ? *reinterpret_cast<const uint4*>(pad + p) : gap;
+  if (t == 0)
+    *reinterpret_cast<uint4*>(sm.code + IX_CHUNK) =
+        q0 + IX_CHUNK < n_pad ? *reinterpret_cast<const uint4*>(pad + q0 + IX_CHUNK) : gap;
+  if (t < IX_BUCKETS) sm.slot[t] = (int32_t)off[t * sh.n_chunks + c];
+  load_classes(sm.cls2, sm.cls3);
+  sm.rank.clear();
+  __syncthreads();
+  const int at0 = warp * (32 * IX_PER) + lane;
+  uint32_t w[IX_PER];  // key << 16 | rank
+#pragma unroll
+  for (int j = 0; j < IX_PER; j++) {
+    const uint32_t b = word_at(sm.code, at0 + 32 * j);
+    const uint32_t a0 = b & 0xff, a1 = b >> 8 & 0xff, a2 = b >> 16 & 0xff, a3 = b >> 24;
+    const bool ok = a0 < NAA && a1 < NAA && a2 < NAA && a3 < NAA;
+    const int key = ok ? (((int)(a0 * 2) + sm.cls2[a1]) * 11 + sm.cls3[a2]) * 20 + (int)a3 : 0;
+    const int r = sm.rank.rank(warp, lane, key >> IX_LO_BITS, ok);
+    w[j] = ok ? (uint32_t)key << 16 | (uint32_t)r : 0xffffffffu;
+  }
+  const int n = sm.rank.scan();
+#pragma unroll
+  for (int j = 0; j < IX_PER; j++)
+    if (w[j] != 0xffffffffu)
+      sm.el[sm.rank.place(warp, (int)(w[j] >> (16 + IX_LO_BITS)), (int)(w[j] & 0xffff))] =
+          w[j] >> 16 << 14 | (uint32_t)(at0 + 32 * j);
+  if (t < IX_BUCKETS) sm.slot[t] -= sm.rank.place(0, t, 0);
+  __syncthreads();
+  for (int i = t; i < n; i += IX_THREADS) {
+    const uint32_t e = sm.el[i];
+    const int slot = sm.slot[e >> (14 + IX_LO_BITS)] + i;
+    by_pos[slot] = (uint32_t)q0 + (e & 0x3fff);
+    by_lo[slot] = (uint8_t)(e >> 14 & (IX_LO - 1));
   }
 }
 
-// Window of indexed word i: cells 0..25 = pad[p .. p+25], cells 26..47 =
-// pad[p-1], pad[p-2], .., pad[p-22]; one thread per window.  The thread reads
-// the 48 bytes S[j] = pad[p - 22 + j] as four aligned 16-byte loads (pad is
-// 16-byte aligned with slack on both sides, so the 64-byte cover stays inside
-// it), selects and funnel-shifts their 12 words into place, and assembles the
-// window: cells 0-25 are S[22..47], cells 26-47 are S[21], S[20], .., S[0].
-// A warp's 32 windows are consecutive in nb: they pass through shared memory
-// and leave as 16-byte stores of consecutive addresses.
-constexpr int NB_THREADS = 256;
-__global__ void __launch_bounds__(NB_THREADS) k_neighbourhoods(const int8_t* pad, const uint32_t* pos, int64_t n,
-                                                               int8_t* nb) {
-  __shared__ uint4 stage[NB_THREADS / 32][32 * 3];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint4* my = stage[warp];
-  for (int64_t w0 = ((int64_t)blockIdx.x * NB_THREADS + warp * 32); w0 < n; w0 += (int64_t)gridDim.x * NB_THREADS) {
-    const int64_t i = w0 + lane;
-    if (i < n) {
-      const int64_t s0 = (int64_t)pos[i] - 22;
-      const int64_t a = s0 & ~(int64_t)15;
-      const int off = (int)(s0 - a), q = off >> 2;
-      const uint32_t sh = 8u * (uint32_t)(off & 3);
-      const uint4* src = reinterpret_cast<const uint4*>(pad + a);
-      uint32_t raw[16];
+// Bound by the shared-memory pipe (84 % of its wavefronts in use; DRAM 35 %,
+// writing 2.9 TB/s): each window passes it twice.  Cutting thirds of windows
+// out of shared memory with three lanes each cost 5.9 wavefronts a word and
+// 3.71 ms where this costs 3.11 (with match.any ranks; 2.96 with ballots).
+//
+// One bucket's words of one group, FILL_CHUNK at a time: sorted by the low
+// digit, a key's words leave as one run of consecutive slots.  The window of
+// a word at p is cells 0..25 = pad[p .. p+25] and 26..47 = pad[p-1], pad[p-2],
+// .., pad[p-22]; with S[j] = pad[p - 22 + j] that is S[22..47] and S[21] ..
+// S[0].  Four lanes fetch the 64 aligned bytes around S (pad is 16-byte
+// aligned with slack on both sides, so they stay inside it) into the warp's
+// corner of shared memory, one lane shifts the window out of them, and the
+// warp's 32 windows leave as 16-byte stores, consecutive within a key's run.
+constexpr int FILL_THREADS = 256;
+constexpr int FILL_WARPS = FILL_THREADS / 32;
+constexpr int FILL_PER = 8;
+constexpr int FILL_CHUNK = FILL_THREADS * FILL_PER;  // 2048
+// 32-bit words a window's bytes take in the corner: 16 and 4, so that rows
+// four apart differ by 16 banks (a quarter warp stores two such rows at once)
+// and the rows a quarter warp reads, one a lane, lie in different banks
+constexpr int FILL_ROW = 20;
+struct FillSmem {
+  uint32_t pos[FILL_CHUNK];
+  uint8_t lo[FILL_CHUNK];
+  alignas(16) uint32_t corner[FILL_WARPS][32 * FILL_ROW];
+  int32_t slot[IX_LO];                               // next slot of each key, less the index of its first word
+  RankSmem<FILL_WARPS> rank;
+};
+static_assert(sizeof(FillSmem) <= 48 * 1024, "static shared memory");
+
+__global__ void __launch_bounds__(FILL_THREADS, 4) k_index_fill(const int8_t* pad, IndexShape sh, const int64_t* off,
+                                                                const uint32_t* by_pos, const uint8_t* by_lo,
+                                                                uint32_t* pos, int8_t* nb) {
+  __shared__ FillSmem sm;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int64_t g = blockIdx.x / IX_BUCKETS;
+  const int b = (int)(blockIdx.x - g * IX_BUCKETS);
+  // the next group's first slot ends this one's (the last group's: the next
+  // bucket's first slot, or the total, which is where the key table starts)
+  const int64_t cell = b * sh.n_chunks + g * sh.group, cell_end = b * sh.n_chunks + min((g + 1) * sh.group, sh.n_chunks);
+  const int64_t i0 = off[cell], i1 = off[cell_end];
+  if (i0 == i1) return;
+  const int64_t* off_key = off + IX_BUCKETS * sh.n_chunks;
+  if (t < IX_LO) {
+    const int64_t k = b * IX_LO + t;
+    sm.slot[t] = k < NKEYS ? (int32_t)(off_key[k * sh.n_groups + g] - off_key[0]) : 0;
+  }
+  for (int64_t c0 = i0; c0 < i1; c0 += FILL_CHUNK) {
+    const int n = (int)min((int64_t)FILL_CHUNK, i1 - c0);
+    const int steps = (n + FILL_THREADS - 1) / FILL_THREADS;  // each warp's share of the words, in 32s
+    const int at0 = warp * 32 * steps + lane;
+    sm.rank.clear();
+    uint32_t p[FILL_PER], w[FILL_PER];  // position; rank << 8 | low digit
 #pragma unroll
-      for (int c = 0; c < 4; c++) {
-        const uint4 v = __ldg(src + c);
-        raw[4 * c] = v.x;
-        raw[4 * c + 1] = v.y;
-        raw[4 * c + 2] = v.z;
-        raw[4 * c + 3] = v.w;
+    for (int j = 0; j < FILL_PER; j++) {
+      const bool ok = j < steps && at0 + 32 * j < n;
+      p[j] = ok ? by_pos[c0 + at0 + 32 * j] : 0;
+      w[j] = ok ? by_lo[c0 + at0 + 32 * j] : IX_LO;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < FILL_PER; j++)
+      if (j < steps) w[j] |= (uint32_t)sm.rank.rank(warp, lane, (int)w[j] & (IX_LO - 1), w[j] < IX_LO) << 8;
+    sm.rank.scan();
+#pragma unroll
+    for (int j = 0; j < FILL_PER; j++)
+      if (!(w[j] & IX_LO)) {
+        const int at = sm.rank.place(warp, (int)(w[j] & 0xff), (int)(w[j] >> 8));
+        sm.pos[at] = p[j];
+        sm.lo[at] = (uint8_t)w[j];
       }
-      uint32_t W[13], S[12];
+    if (t < IX_LO) sm.slot[t] -= sm.rank.place(0, t, 0);
+    __syncthreads();
+    for (int i = t; i < n; i += FILL_THREADS) pos[sm.slot[sm.lo[i]] + i] = sm.pos[i];
+    uint32_t* corner = sm.corner[warp];
+    // the row and quarter of this lane's fetches, and where they are kept
+    const int frow = (lane >> 3) + (lane & 4), quarter = lane & 3;
+    for (int i = 32 * warp; i < n; i += FILL_THREADS) {
+      uint4 v[4];
 #pragma unroll
-      for (int k = 0; k < 13; k++) W[k] = q == 0 ? raw[k] : q == 1 ? raw[k + 1] : q == 2 ? raw[k + 2] : raw[k + 3];
+      for (int r = 0; r < 4; r++) {
+        const int x = min(i + 8 * r + frow, n - 1);
+        v[r] = __ldg(reinterpret_cast<const uint4*>(pad + (((int64_t)sm.pos[x] - 22) & ~(int64_t)15)) + quarter);
+      }
 #pragma unroll
-      for (int k = 0; k < 12; k++) S[k] = __funnelshift_r(W[k], W[k + 1], sh);
-      uint32_t o[12];
+      for (int r = 0; r < 4; r++)
+        *reinterpret_cast<uint4*>(corner + (8 * r + frow) * FILL_ROW + 4 * quarter) = v[r];
+      __syncwarp();
+      const int x = min(i + lane, n - 1);
+      const uint32_t o = (sm.pos[x] - 22) & 15;
+      uint32_t raw[16], W[13], S[12], cell[12];
 #pragma unroll
-      for (int k = 0; k < 6; k++) o[k] = __funnelshift_r(S[5 + k], S[6 + k], 16);  // S[22 + 4k ..]
-      o[6] = __byte_perm(S[11], S[5], 0x4532u);                                   // S46 S47 S21 S20
+      for (int k = 0; k < 4; k++) {
+        const uint4 r = *reinterpret_cast<const uint4*>(corner + lane * FILL_ROW + 4 * k);
+        raw[4 * k] = r.x, raw[4 * k + 1] = r.y, raw[4 * k + 2] = r.z, raw[4 * k + 3] = r.w;
+      }
+      const bool two = o & 8, one = o & 4;
 #pragma unroll
-      for (int k = 7; k < 12; k++) o[k] = __byte_perm(S[11 - k], 0u, 0x0123u);    // S[4(11-k)+3] .. S[4(11-k)]
-      my[3 * lane] = make_uint4(o[0], o[1], o[2], o[3]);
-      my[3 * lane + 1] = make_uint4(o[4], o[5], o[6], o[7]);
-      my[3 * lane + 2] = make_uint4(o[8], o[9], o[10], o[11]);
+      for (int k = 0; k < 14; k++) raw[k] = two ? raw[k + 2] : raw[k];
+#pragma unroll
+      for (int k = 0; k < 13; k++) W[k] = one ? raw[k + 1] : raw[k];
+#pragma unroll
+      for (int k = 0; k < 12; k++) S[k] = __funnelshift_r(W[k], W[k + 1], 8 * (o & 3));  // S[4k ..]
+#pragma unroll
+      for (int k = 0; k < 6; k++) cell[k] = __funnelshift_r(S[5 + k], S[6 + k], 16);     // S[22 + 4k ..]
+      cell[6] = __byte_perm(S[11], S[5], 0x4532);                                        // S46 S47 S21 S20
+#pragma unroll
+      for (int k = 7; k < 12; k++) cell[k] = __byte_perm(S[11 - k], 0, 0x0123);          // S[4(11-k)+3] .. S[4(11-k)]
+      __syncwarp();
+      uint4* out = reinterpret_cast<uint4*>(corner);
+      out[3 * lane] = make_uint4(cell[0], cell[1], cell[2], cell[3]);
+      out[3 * lane + 1] = make_uint4(cell[4], cell[5], cell[6], cell[7]);
+      out[3 * lane + 2] = make_uint4(cell[8], cell[9], cell[10], cell[11]);
+      const int slot = sm.slot[sm.lo[x]] + x;
+      __syncwarp();
+#pragma unroll
+      for (int r = 0; r < 3; r++) {
+        const int e = 32 * r + lane, row = e / 3;
+        const int64_t to = __shfl_sync(0xffffffffu, slot, row);
+        if (i + row < n) *reinterpret_cast<uint4*>(nb + to * WIN + 16 * (e - 3 * row)) = out[e];
+      }
+      __syncwarp();
     }
-    __syncwarp();
-    const int cnt = (int)min((int64_t)32, n - w0);
-    uint4* dst = reinterpret_cast<uint4*>(nb + w0 * WIN);
-#pragma unroll
-    for (int r = 0; r < 3; r++) {
-      const int e = lane + 32 * r;
-      if (e < 3 * cnt) dst[e] = my[e];
-    }
-    __syncwarp();
+    __syncthreads();
+    // a key's next word follows this chunk's last: its first word's index
+    // back on, and the count (the next digit's first place less its own)
+    if (t < IX_LO) sm.slot[t] += t + 1 < IX_LO ? sm.rank.place(0, t + 1, 0) : n;
+    __syncthreads();
   }
 }
 
@@ -401,53 +560,48 @@ cudaError_t launch_build_pad(const int8_t* codes, const int64_t* seq_off, int32_
   return cudaGetLastError();
 }
 
-int64_t index_tile(int64_t n_pad) {
-  // about six one-warp CTAs on each of 152 SMs
-  int64_t t = (n_pad + 912 - 1) / 912;
-  t = (t + IX_CHUNK - 1) / IX_CHUNK * IX_CHUNK;
-  return std::min<int64_t>(std::max<int64_t>(t, IX_CHUNK), 16 * IX_CHUNK);
+IndexShape index_shape(int64_t n_pad) {
+  IndexShape sh;
+  sh.n_chunks = (n_pad + IX_CHUNK - 1) / IX_CHUNK;
+  // four CTAs of k_index_hist an SM before one takes more than one chunk
+  sh.per = 1;
+  while (sh.per < 8 && sh.n_chunks / (2 * sh.per) >= 608) sh.per *= 2;
+  // 18 groups or more keep 152 SMs busy with a bucket each; a group of 64
+  // chunks gives each of its 69 buckets some 6,000 words
+  sh.group = std::min<int64_t>(64, std::max<int64_t>(1, sh.n_chunks / 18));
+  sh.group = (sh.group + sh.per - 1) / sh.per * sh.per;
+  sh.n_groups = (sh.n_chunks + sh.group - 1) / sh.group;
+  return sh;
 }
 
-cudaError_t launch_index_hist(const int8_t* pad, int64_t n_pad, int64_t tile, int64_t n_tiles, int32_t* hist,
+int64_t index_cells(const IndexShape& sh) { return IX_BUCKETS * sh.n_chunks + (int64_t)NKEYS * sh.n_groups; }
+
+cudaError_t launch_index_hist(const int8_t* pad, int64_t n_pad, const IndexShape& sh, int32_t* hist,
                               cudaStream_t st) {
-  if (n_tiles > 0) {
-    note_launch();
-    k_index_hist<<<(unsigned)n_tiles, IX_THREADS, 0, st>>>(pad, n_pad, tile, n_tiles, hist);
-  }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_index_finish(const int8_t* pad, int64_t n_pad, int64_t tile, int64_t n_tiles, const int64_t* off,
-                                int64_t* offT, const int64_t* total, int64_t* key_off, uint32_t* pos,
-                                cudaStream_t st) {
-  // one-warp CTAs with 35 KB of shared memory each: ask for the largest
-  // shared-memory carveout so that six of them share an SM
-  static std::atomic<bool> carveout_set[64];  // per device; calls may come from several threads
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev < 64 && !carveout_set[dev]) {
-    cudaError_t e = cudaFuncSetAttribute(k_index_scatter, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                         (int)cudaSharedmemCarveoutMaxShared);
-    if (e != cudaSuccess) return e;
-    carveout_set[dev] = true;
-  }
+  cudaError_t e = cudaMemsetAsync(hist + IX_BUCKETS * sh.n_chunks, 0, (size_t)NKEYS * sh.n_groups * sizeof(int32_t), st);
+  if (e != cudaSuccess) return e;
   note_launch();
-  k_index_key_off<<<(NKEYS + 1 + 255) / 256, 256, 0, st>>>(off, n_tiles, total, key_off);
-  if (n_tiles > 0) {
-    note_launch();
-    k_index_transpose<<<dim3((unsigned)((n_tiles + 31) / 32), (NKEYS + 31) / 32), dim3(32, 8), 0, st>>>(off, n_tiles,
-                                                                                                     offT);
-    note_launch();
-    k_index_scatter<<<(unsigned)n_tiles, 32, 0, st>>>(pad, n_pad, tile, offT, pos);
-  }
+  k_index_hist<<<(unsigned)((sh.n_chunks + sh.per - 1) / sh.per), IX_THREADS, 0, st>>>(pad, n_pad, sh, hist);
   return cudaGetLastError();
 }
 
-cudaError_t launch_neighbourhoods(const int8_t* pad, const uint32_t* pos, int64_t n, int8_t* nb, cudaStream_t st) {
-  if (n > 0) {
-    note_launch();
-    k_neighbourhoods<<<grid_for(n, NB_THREADS), NB_THREADS, 0, st>>>(pad, pos, n, nb);
-  }
+cudaError_t launch_index_key_off(const int64_t* off, const IndexShape& sh, int64_t* key_off, cudaStream_t st) {
+  note_launch();
+  k_index_key_off<<<(NKEYS + 1 + 255) / 256, 256, 0, st>>>(off, sh, key_off);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_index_split(const int8_t* pad, int64_t n_pad, const IndexShape& sh, const int64_t* off,
+                               uint32_t* by_pos, uint8_t* by_lo, cudaStream_t st) {
+  note_launch();
+  k_index_split<<<(unsigned)sh.n_chunks, IX_THREADS, 0, st>>>(pad, n_pad, sh, off, by_pos, by_lo);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_index_fill(const int8_t* pad, const IndexShape& sh, const int64_t* off, const uint32_t* by_pos,
+                              const uint8_t* by_lo, uint32_t* pos, int8_t* nb, cudaStream_t st) {
+  note_launch();
+  k_index_fill<<<(unsigned)(sh.n_groups * IX_BUCKETS), FILL_THREADS, 0, st>>>(pad, sh, off, by_pos, by_lo, pos, nb);
   return cudaGetLastError();
 }
 
