@@ -150,6 +150,16 @@ int num_sms() {
 // the plain wide kernel, which runs at an S1 below UNG_TC_MIN_S1, is charged
 // PLAIN_WIDE_SLOT for every row of the shape.
 constexpr int TC_FIXED_ROWS = 83;
+// A key's rest goes to the tensor kernel where that costs less than
+// NARROW_SHARE of the narrow tiles' charge (in a whole launch these come to
+// 0.85 - 0.9 of it: 187 x 70,000 proteins on narrow tiles alone are charged
+// 1.06 ms and take 0.93), and if no key fills a wide tile only when all rests
+// together save the launch and its ramps, WIDE_LAUNCH ns on every SM.
+// Measured, stage 2, rests by plain cost / by this rule / the better of that
+// and narrow tiles alone: 90 x 70,000 0.565 / 0.536 / 0.534 ms, 187 x 200,000
+// 2.575 / 2.48 / 2.48, 250 x 200,000 3.03 / 3.01 / 3.01, 400 x 70,000 1.459 /
+// 1.467 / 1.459 (narrow alone 1.77).
+constexpr double NARROW_SHARE = 0.87, WIDE_LAUNCH = 30000.0;
 constexpr double PLAIN_WIDE_SLOT = 0.317, PLAIN_WIDE_TILE = 2960.0;
 std::mutex g_cost_mu;
 plast_tile_costs g_costs = {0.140, 3660.0, 0.479, 566.0, 0.616, 1101.0, 1.094, 1090.0, 12, 0, 0.416, 314.0};
@@ -271,7 +281,8 @@ void split_long_tiles(const plast_tile_costs& c, std::vector<int4>& v, int64_t l
 }
 
 void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first, TileList* tl,
-                      const std::vector<char>* key_mask, int shape_override, int n_sms, bool tensor, bool listed = false) {
+                      const std::vector<char>* key_mask, int shape_override, int n_sms, bool tensor,
+                      bool listed = false, bool narrow_rests = false) {
   tl->tiles.clear();
   tl->tensor = tensor;
   tl->pairs = 0;
@@ -339,6 +350,8 @@ void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first
   double best[TAIL];
   int pick[TAIL];
   int64_t cover_passes = -1;
+  double rests_gain = 0;  // of the keys' rests as wide tiles, over narrow ones
+  bool full_wide = false;
   auto emit = [&](int k, int64_t first, int64_t rows, int shape) {
     const int4 t = make_tile(k, (int)first, (int)rows, shape, 0, n2_now);
     if (out) out->push_back(t);
@@ -358,7 +371,10 @@ void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first
       for (; u < end; u += r) emit(k, u, std::min<int64_t>(r, end - u), shape);
       continue;
     }
-    for (; end - u >= UNG_T1; u += UNG_T1) emit(k, u, UNG_T1, UNG_WIDE);
+    for (; end - u >= UNG_T1; u += UNG_T1) {
+      emit(k, u, UNG_T1, UNG_WIDE);
+      full_wide = true;
+    }
     const int64_t rem = end - u;
     if (rem <= 0) continue;
     if (mode == 1) {
@@ -385,7 +401,10 @@ void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first
     const int64_t full = rem / br;
     const int tail = (int)(rem % br);
     const double narrow_cost = (double)full * cost_now[bulk] + best[tail];
-    if (!(narrow_cost < tile_cost(c, UNG_WIDE, n2, tensor ? rem : UNG_T1))) {
+    const double wide_cost = tile_cost(c, UNG_WIDE, n2, tensor ? rem : UNG_T1);
+    const double gain = (tensor ? NARROW_SHARE * narrow_cost : narrow_cost) - wide_cost;
+    if (!narrow_rests && gain >= 0) {
+      rests_gain += gain;
       emit(k, u, rem, UNG_WIDE);
       continue;
     }
@@ -396,6 +415,10 @@ void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first
       u += r;
       t -= r;
     }
+  }
+  if (tensor && mode == 0 && n_sms > 0 && rests_gain > 0 && !full_wide && rests_gain < WIDE_LAUNCH * n_sms) {
+    build_tiles_from(ko1, ko2, largest_first, tl, key_mask, shape_override, n_sms, tensor, listed, true);
+    return;
   }
   if (!largest_first) {
     for (const int4& t : tl->tiles) tl->n_wide += tile_shape(t) == UNG_WIDE;
