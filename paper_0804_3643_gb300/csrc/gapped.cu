@@ -8,10 +8,11 @@
 // holding the two sides of the same hits are adjacent lanes and add their
 // sides with shuffles.  CTAs stride over the hits.
 //
-// Per cell (two hits): two byte loads of B_j from the thread's shared
-// segments, two IMADs and two loads of s(A_i, B_j) - go from a lane-replicated
+// Per cell (two hits): two loads of s(A_i, B_j) - go from a lane-replicated
 // table (entry (a, b) of lane l at word (b * 23 + a) * 32 + l: the lanes of a
-// warp never share a bank), one IMAD packing the two entries, then four
+// warp never share a bank), their addresses from one two-way dot product each
+// (the row's address plus one half of a register that holds the table offsets
+// of both hits' B_j), one IMAD packing the two entries, then four
 // three-operand maxima.  Row i's values are kept offset by i * ge, and F and
 // DF also shifted down by goe = go + ge:
 //   H'  = H + i ge,  E' = E + i ge,  Gg = F + i ge - goe,  DFg = DF + i ge - goe
@@ -43,10 +44,20 @@
 // through a sentinel cell comes back above the best cell of the clipped
 // grid, so the fixed band over i <= LG equals the one clipped at the sequence
 // ends.  Columns j < 0 start at -16000 and stay far below zero.  Columns
-// j > LG (rows i > LG - BAND) lie outside the grid and feed no cell of it
-// (a cell reads only cells of its own or a smaller column), so they are not
-// computed (compile-time column limits); the stale values left in their
-// slots are read only by other such cells.
+// j > LG (rows i > LG - BAND) lie outside the grid: they are staged as
+// sentinels, so a cell there is at most the cell of the grid its path left
+// from, in its own row or an earlier one, whatever the gap costs (they may be
+// 0): it never raises the best value, and the end column is looked for on the
+// grid only.
+//
+// Bound by the rate of three-operand instructions: of 13.3 instructions a
+// cell 9 read three registers, and a loop of the same mix on registers alone
+// takes 17.3 clocks a cell per warp and scheduler where this takes 18.1.
+// Four rows share their B offsets in registers, and all 64 rows run through
+// one loop of four (15 KB of code; eight rows unrolled do not fit the
+// instruction cache: 23.3 ms, two rows move more registers: 19.5): 18.6 ms for
+// the 37.5 M hits of 10,000 x 100,000 proteins.  A byte load per cell and the
+// last eight rows unrolled with only their grid columns took 19.05.
 #include <atomic>
 
 #include "gapped.cuh"
@@ -58,8 +69,10 @@ namespace plast {
 constexpr int NEG16 = -16000;
 constexpr int GAP_THREADS = 256;
 constexpr int TAB_A = 23;                                   // padded entries per b
+constexpr int B_STRIDE = TAB_A * 32 * 4;                    // bytes from one b to the next
+static_assert((NCODE - 1) * B_STRIDE < 1 << 16, "the offset of a b fits a half word");
 constexpr int TAB_WORDS = NCODE * TAB_A * 32;               // lane-replicated
-constexpr int SEG_W = 22;                                   // words staged per hit: B_-8 .. B_74 + slack
+constexpr int SEG_W = 22;                                   // words staged per hit: B_-8 .. B_79
 constexpr int SEG_B = SEG_W * 4;                            // 88 bytes
 constexpr int SEG_T = 2 * SEG_B + 4;                        // 45 words per thread: odd, no bank conflict
 constexpr int GAP_SMEM = TAB_WORDS * 4 + GAP_THREADS * SEG_T;  // 110848 bytes
@@ -76,13 +89,38 @@ struct GapConst {
   int ge;
 };
 
-// Cell JB of row i for both hits.
+// Table offsets of B_{i - BAND} .. B_{i + BAND + 3} of both hits (low and high
+// half), i the first row of a group of four: row i + r takes X[r + jb] for its
+// cell jb.
+struct Cols {
+  uint32_t X[BW + 3];
+  // entries K .. BW + 2 from the segments (sb0, sb1: B_{i - BAND})
+  template <int K>
+  __device__ __forceinline__ void load(uint32_t sb0, uint32_t sb1) {
+    if constexpr (K < BW + 3) {
+      X[K] = lds_u8<K>(sb0) * (uint32_t)B_STRIDE + lds_u8<K>(sb1) * ((uint32_t)B_STRIDE << 16);
+      load<K + 1>(sb0, sb1);
+    }
+  }
+  __device__ __forceinline__ void next(uint32_t sb0, uint32_t sb1) {
+#pragma unroll
+    for (int k = 0; k < BW - 1; k++) X[k] = X[k + 4];
+    load<BW - 1>(sb0, sb1);
+  }
+};
+
+__device__ __forceinline__ uint32_t lds_u32(uint32_t at) {
+  uint32_t v;
+  asm("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(at));
+  return v;
+}
+
+// Cell JB of row i for both hits; row0, row1: the table's rows of A_i.
 template <int JB>
-__device__ __forceinline__ uint32_t band_cell(Band& B, const unsigned char* row0, const unsigned char* row1,
-                                              uint32_t sb0, uint32_t sb1, uint32_t& E, const GapConst& k) {
-  const uint32_t b0 = lds_u8<JB>(sb0), b1 = lds_u8<JB>(sb1);  // B_{i - BAND + JB} of each hit
-  const uint32_t s0 = *reinterpret_cast<const uint32_t*>(row0 + b0 * (TAB_A * 128));
-  const uint32_t s1 = *reinterpret_cast<const uint32_t*>(row1 + b1 * (TAB_A * 128));
+__device__ __forceinline__ void band_cell(Band& B, uint32_t row0, uint32_t row1, uint32_t x, uint32_t& E,
+                                          const GapConst& k) {
+  const uint32_t s0 = lds_u32(__dp2a_lo(x, 0x0001u, row0));  // row0 + the low half of x
+  const uint32_t s1 = lds_u32(__dp2a_lo(x, 0x0100u, row1));  // row1 + the high half
   const uint32_t sc = s1 * 65536u + s0;  // entries are zero-extended int16 s - go
   const uint32_t up_h = JB + 1 < BW ? B.H[JB + 1 < BW ? JB + 1 : 0] : x2(NEG16);
   const uint32_t up_g = JB + 1 < BW ? B.Gg[JB + 1 < BW ? JB + 1 : 0] : x2(NEG16);
@@ -92,35 +130,29 @@ __device__ __forceinline__ uint32_t band_cell(Band& B, const unsigned char* row0
   E = __viaddmax_s16x2(E, k.nge2, dfg);                        // E' of the next cell
   B.H[JB] = h;
   B.Gg[JB] = gg;
-  return h;
 }
 
-// Cells 0 .. JLIM of row i (the cells JB > JLIM have j > LG, see below).
-template <int JB, int JLIM>
-__device__ __forceinline__ void band_cells(Band& B, const unsigned char* row0, const unsigned char* row1,
-                                           uint32_t sb0, uint32_t sb1, uint32_t& E, const GapConst& k) {
-  if constexpr (JB <= JLIM) {
-    band_cell<JB>(B, row0, row1, sb0, sb1, E, k);
-    band_cells<JB + 1, JLIM>(B, row0, row1, sb0, sb1, E, k);
+// The cells of row R of its group.
+template <int JB, int R>
+__device__ __forceinline__ void band_cells(Band& B, uint32_t row0, uint32_t row1, const Cols& c, uint32_t& E,
+                                           const GapConst& k) {
+  if constexpr (JB < BW) {
+    band_cell<JB>(B, row0, row1, c.X[JB + R], E, k);
+    band_cells<JB + 1, R>(B, row0, row1, c, E, k);
   }
 }
 
-// Maximum of H'[0 .. JLIM], three at a time.
-template <int JB, int JLIM>
-__device__ __forceinline__ uint32_t row_max(const Band& B, uint32_t m) {
-  if constexpr (JB + 1 <= JLIM) return row_max<JB + 2, JLIM>(B, __vimax3_s16x2(m, B.H[JB], B.H[JB + 1]));
-  else if constexpr (JB <= JLIM) return __vmaxs2(m, B.H[JB]);
-  else return m;
-}
-
-// Row i; columns jb > JLIM have j > LG: they are neither computed nor in the
-// maximum.
-template <int JLIM>
-__device__ __forceinline__ void gapped_row(Band& B, int i, const unsigned char* row0, const unsigned char* row1,
-                                           uint32_t sb0, uint32_t sb1, const GapConst& k) {
+// Row i, the R-th of its group.
+template <int R>
+__device__ __forceinline__ void gapped_row(Band& B, int i, uint32_t row0, uint32_t row1, const Cols& c,
+                                           const GapConst& k) {
+  static_assert(BW % 2 == 1, "the row maximum takes two columns at a time");
   uint32_t E = x2(NEG16);
-  band_cells<0, JLIM>(B, row0, row1, sb0 + i, sb1 + i, E, k);
-  const uint32_t rmax = __vsub2(row_max<1, JLIM>(B, B.H[0]), x2(i * k.ge));  // without the row offset
+  band_cells<0, R>(B, row0, row1, c, E, k);
+  uint32_t rmax = B.H[0];
+#pragma unroll
+  for (int jb = 1; jb < BW; jb += 2) rmax = __vimax3_s16x2(rmax, B.H[jb], B.H[jb + 1]);
+  rmax = __vsub2(rmax, x2(i * k.ge));            // without the row offset
   const uint32_t up = __vcmpgts2(rmax, B.best);  // 0xffff in the halves that improve
   B.best = __vmaxs2(B.best, rmax);
   B.bi = (x2(i) & up) | (B.bi & ~up);
@@ -141,12 +173,13 @@ __device__ __forceinline__ int end_column(const Band& B, int q, int ge) {
   return bi - BAND + found;
 }
 
-// Copy B_-8 .. B_74 of one hit side into a thread's segment in reading
+// Copy B_-8 .. B_64 of one hit side into a thread's segment in reading
 // order with aligned 32-bit loads, B_-8 landing on the segment's first byte
 // (so the byte loads of a warp stay conflict-free); returns its shared address.
 // Right side: B_j = pad2[p2 + j - 1], the bytes [p2 - 9, p2 + 73] forwards.
 // Left side:  B_j = pad2[p2 - j],     the bytes [p2 - 74, p2 + 8] backwards,
 // each word byte-reversed.
+// B_65 on (byte 73 on) are sentinels: those columns lie outside the grid.
 __device__ __forceinline__ uint32_t stage_b(const int8_t* pad2, int64_t p2, int side, uint32_t* dst,
                                             uint32_t dst_s) {
   const int64_t lo = p2 - 9, hi = p2 + BAND;
@@ -154,11 +187,18 @@ __device__ __forceinline__ uint32_t stage_b(const int8_t* pad2, int64_t p2, int 
   const uint32_t sel = side ? 0x0123u : 0x3210u;
   const uint32_t sh = 8u * (side ? (uint32_t)(3 - (hi & 3)) : (uint32_t)(lo & 3));
   const uint32_t* src = reinterpret_cast<const uint32_t*>(pad2 + first);
+  constexpr int B65 = BAND + LG + 1;  // byte of B_65
+  static_assert(B65 % 4 == 1, "one byte of its word lies on the grid");
   uint32_t w[SEG_W + 1];
 #pragma unroll
   for (int k = 0; k <= SEG_W; k++) w[k] = __byte_perm(__ldg(src + (side ? -k : k)), 0u, sel);
 #pragma unroll
-  for (int k = 0; k < SEG_W; k++) dst[k] = __funnelshift_r(w[k], w[k + 1], sh);
+  for (int k = 0; k < SEG_W; k++) {
+    uint32_t v = __funnelshift_r(w[k], w[k + 1], sh);
+    if (k == B65 / 4) v = __byte_perm(v, 0x01010101u * SENTINEL, 0x7650u);
+    if (k > B65 / 4) v = 0x01010101u * SENTINEL;
+    dst[k] = v;
+  }
   return dst_s;
 }
 
@@ -198,7 +238,7 @@ __global__ void __launch_bounds__(GAP_THREADS, 2) k_small_gapped(GapArgs a) {
     tab32[e * 32 + lane] = aa < NCODE ? (uint32_t)(uint16_t)(int16_t)(c_score[aa * NCODE + b] - go) : 0u;
   }
   __syncthreads();
-  const unsigned char* tlane = reinterpret_cast<const unsigned char*>(tab32) + lane * 4;
+  const uint32_t tlane = (uint32_t)__cvta_generic_to_shared(tab32) + lane * 4;
   GapConst kc;
   kc.nge2 = x2(-ge);
   kc.goe2 = x2(goe);
@@ -222,7 +262,7 @@ __global__ void __launch_bounds__(GAP_THREADS, 2) k_small_gapped(GapArgs a) {
       const int64_t p11 = (int64_t)(k1 >> a.sh), p21 = (int64_t)(k1 & mask);
       // residue i (1-based): right A_i = pad1[p1 + i - 1], B_j = pad2[p2 + j - 1];
       // left A_i = pad1[p1 - i], B_j = pad2[p2 - j].
-      // B_-8 .. B_74 of each hit in reading order: aligned words of pad2,
+      // B_-8 .. B_64 of each hit in reading order: aligned words of pad2,
       // taken backwards and byte-reversed for the left side; sbX points at B_-8
       const uint32_t sb0 = stage_b(a.pad2, p20, side, reinterpret_cast<uint32_t*>(seg), seg_s);
       const uint32_t sb1 = stage_b(a.pad2, p21, side, reinterpret_cast<uint32_t*>(seg + SEG_B), seg_s + SEG_B);
@@ -243,37 +283,25 @@ __global__ void __launch_bounds__(GAP_THREADS, 2) k_small_gapped(GapArgs a) {
       ra0.init(a.pad1, p10 - side, side);
       ra1.init(a.pad1, p11 - side, side);
       uint32_t aw0 = ra0.next(), aw1 = ra1.next();
-#define PLAST_ROW(I, R, JLIM)                                                                          \
+      Cols cols;
+      cols.load<4>(sb0 - 3, sb1 - 3);
+#define PLAST_ROW(I, R)                                                                                \
   {                                                                                                    \
-    const unsigned char* r0 = tlane + __byte_perm(c0, 0u, 0x4440u + (R)) * 128u;                       \
-    const unsigned char* r1 = tlane + __byte_perm(c1, 0u, 0x4440u + (R)) * 128u;                       \
-    gapped_row<JLIM>(B, (I), r0, r1, sb0, sb1, kc);                                                    \
+    const uint32_t r0 = tlane + __byte_perm(c0, 0u, 0x4440u + (R)) * 128u;                             \
+    const uint32_t r1 = tlane + __byte_perm(c1, 0u, 0x4440u + (R)) * 128u;                             \
+    gapped_row<R>(B, (I), r0, r1, cols, kc);                                                     \
   }
-      for (int g = 0; g < (LG - BAND) / 4; g++) {  // rows 1 .. 56: the whole band on the grid
+      #pragma unroll 1
+      for (int g = 0; g < LG / 4; g++) {
         const uint32_t c0 = aw0, c1 = aw1;
         aw0 = ra0.next();
         aw1 = ra1.next();
         const int i = 4 * g + 1;
-        PLAST_ROW(i, 0, BW - 1)
-        PLAST_ROW(i + 1, 1, BW - 1)
-        PLAST_ROW(i + 2, 2, BW - 1)
-        PLAST_ROW(i + 3, 3, BW - 1)
-      }
-      {  // rows 57 .. 60
-        const uint32_t c0 = aw0, c1 = aw1;
-        aw0 = ra0.next();
-        aw1 = ra1.next();
-        PLAST_ROW(LG - BAND + 1, 0, 15)
-        PLAST_ROW(LG - BAND + 2, 1, 14)
-        PLAST_ROW(LG - BAND + 3, 2, 13)
-        PLAST_ROW(LG - BAND + 4, 3, 12)
-      }
-      {  // rows 61 .. 64
-        const uint32_t c0 = aw0, c1 = aw1;
-        PLAST_ROW(LG - BAND + 5, 0, 11)
-        PLAST_ROW(LG - BAND + 6, 1, 10)
-        PLAST_ROW(LG - BAND + 7, 2, 9)
-        PLAST_ROW(LG - BAND + 8, 3, 8)
+        cols.next(sb0 + i, sb1 + i);
+        PLAST_ROW(i, 0)
+        PLAST_ROW(i + 1, 1)
+        PLAST_ROW(i + 2, 2)
+        PLAST_ROW(i + 3, 3)
       }
 #undef PLAST_ROW
     } else {
