@@ -227,62 +227,76 @@ int64_t charged_rows(const int4& t, bool tensor) {
   return tensor && tile_shape(t) == UNG_WIDE ? tile_rows(t) : UNG_T1;
 }
 
+struct PlannedTile {
+  double cost;
+  int4 tile;
+};
+bool costlier(const PlannedTile& x, const PlannedTile& y) { return x.cost > y.cost; }
+
+// The lists that a tile plan goes through, kept by the thread that plans: as
+// fresh vectors their page faults took half of a small search's planning.
+// Given back after a plan of more than a million tiles.
+struct PlanLists {
+  std::vector<PlannedTile> wide, by_shape[UNG_SHAPES], rests[UNG_SHAPES], narrow, half[2], rest, pieces;
+  std::vector<int> keys, sorted;
+  void clear() {
+    size_t held = 0;
+    auto each = [&](std::vector<PlannedTile>& v) {
+      held += v.capacity();
+      v.clear();
+    };
+    for (auto* v : {&wide, &narrow, &half[0], &half[1], &rest, &pieces}) each(*v);
+    for (auto& v : by_shape) each(v);
+    for (auto& v : rests) each(v);
+    if (held > 1 << 20) *this = PlanLists();
+  }
+};
+PlanLists& plan_lists() {
+  static thread_local PlanLists lists;
+  return lists;
+}
+
 // When a launch has too few tiles to keep its CTAs busy to the end (a small
 // query bank: a few hundred keys with one or two bank-1 occurrences), the
 // costliest tiles are cut along their bank-2 lists into pieces of whole
-// passes, so that no piece costs more than about 1/4 of a CTA's share; the
-// pieces re-sorted costliest first.  v[lo, hi) is one launch's tile list.
-void split_long_tiles(const plast_tile_costs& c, std::vector<int4>& v, int64_t lo, int64_t hi, int64_t ctas,
-                      bool tensor) {
-  if (hi <= lo || ctas <= 0) return;
-  auto cost = [&](const int4& t) {
-    return tile_cost(c, tile_shape(t), (int64_t)t.w - t.z, charged_rows(t, tensor));
-  };
-  // the list is costliest first: a tile above twice the target exists only if
-  // the first one is above it, and the target is at most the first tile's
-  // cost times the tile count over 4 * ctas
-  if (hi - lo > 8 * ctas) {
-    const double c0 = cost(v[lo]);
-    double total = 0;
-    for (int64_t i = lo; i < hi; i++) total += cost(v[i]);
-    if (c0 <= 2 * total / (4.0 * (double)ctas)) return;
-  }
-  double total = 0;
-  for (int64_t i = lo; i < hi; i++) total += cost(v[i]);
+// passes, so that no piece costs more than about 1/4 of a CTA's share, and the
+// pieces take their places costliest first.  v is one launch's tile list,
+// costliest first but for the partial wide tiles.
+void split_long_tiles(const plast_tile_costs& c, std::vector<PlannedTile>& v, int64_t ctas, bool tensor) {
+  if (v.empty() || ctas <= 0) return;
+  double total = 0, largest = 0;
+  for (const PlannedTile& t : v) total += t.cost, largest = std::max(largest, t.cost);
   const double target = total / (4.0 * (double)ctas);
-  bool any = false;
-  for (int64_t i = lo; i < hi && !any; i++) any = cost(v[i]) > 2 * target;
-  if (!any) return;
-  std::vector<std::pair<double, int4>> out;
-  out.reserve((size_t)(hi - lo) * 2);
-  for (int64_t i = lo; i < hi; i++) {
-    const int4 t = v[i];
-    const double ct = cost(t);
+  if (largest <= 2 * target) return;
+  std::vector<PlannedTile>&rest = plan_lists().rest, &pieces = plan_lists().pieces;
+  rest.clear();
+  pieces.clear();
+  for (const PlannedTile& x : v) {
+    const int4 t = x.tile;
     const int shape = tile_shape(t);
     const int64_t pass = shape == UNG_WIDE ? WIDE_PASS : NARROW_PASS, n2 = (int64_t)t.w - t.z;
-    const int64_t pieces = std::min<int64_t>((int64_t)std::ceil(ct / target), (n2 + pass - 1) / pass);
-    if (ct <= 2 * target || pieces < 2) {
-      out.push_back({ct, t});
+    const int64_t cuts =
+        x.cost <= 2 * target ? 1 : std::min<int64_t>((int64_t)std::ceil(x.cost / target), (n2 + pass - 1) / pass);
+    if (cuts < 2) {
+      rest.push_back(x);
       continue;
     }
-    const int64_t chunk = round_up((n2 + pieces - 1) / pieces, pass);
+    const int64_t chunk = round_up((n2 + cuts - 1) / cuts, pass);
     for (int64_t a = 0; a < n2; a += chunk) {
       const int4 p = make_tile(tile_key(t), t.y, tile_rows(t), shape, t.z + (int)a,
                                t.z + (int)std::min<int64_t>(a + chunk, n2));
-      out.push_back({cost(p), p});
+      pieces.push_back({tile_cost(c, shape, (int64_t)p.w - p.z, charged_rows(p, tensor)), p});
     }
   }
-  std::stable_sort(out.begin(), out.end(),
-                   [](const std::pair<double, int4>& x, const std::pair<double, int4>& y) { return x.first > y.first; });
-  std::vector<int4> nv(v.begin(), v.begin() + lo);
-  for (const auto& x : out) nv.push_back(x.second);
-  nv.insert(nv.end(), v.begin() + hi, v.end());
-  v.swap(nv);
+  if (!std::is_sorted(rest.begin(), rest.end(), costlier)) std::stable_sort(rest.begin(), rest.end(), costlier);
+  std::stable_sort(pieces.begin(), pieces.end(), costlier);
+  v.resize(rest.size() + pieces.size());
+  std::merge(rest.begin(), rest.end(), pieces.begin(), pieces.end(), v.begin(), costlier);
 }
 
 void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first, TileList* tl,
                       const std::vector<char>* key_mask, int shape_override, int n_sms, bool tensor,
-                      bool listed = false, bool narrow_rests = false) {
+                      bool listed = false) {
   tl->tiles.clear();
   tl->tensor = tensor;
   tl->pairs = 0;
@@ -300,8 +314,10 @@ void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first
   // Keys in launch order: the persistent schedule takes them by decreasing
   // n2, which orders the tiles of each shape by decreasing cost (a tile's
   // cost depends on its shape and n2 only), so the tiles need no sort.
-  std::vector<int> keys;
-  keys.reserve(NKEYS);
+  PlanLists& lists = plan_lists();
+  lists.clear();
+  std::vector<int>& keys = lists.keys;
+  keys.clear();
   for (int k = 0; k < NKEYS; k++) {
     if (key_mask && !(*key_mask)[k]) continue;
     if (ko1[k + 1] == ko1[k] || ko2[k + 1] == ko2[k]) continue;
@@ -321,26 +337,16 @@ void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first
     };
     for (const int k : keys) count[bucket(k) + 1]++;
     for (int b = 0; b < NB; b++) count[b + 1] += count[b];
-    std::vector<int> sorted(keys.size());
+    std::vector<int>& sorted = lists.sorted;
+    sorted.resize(keys.size());
     for (const int k : keys) sorted[count[bucket(k)]++] = k;
     keys.swap(sorted);
   }
   // wide tiles, then narrow tiles of 16, 8, 4 and 2 rows, each in key order
   // (narrow tiles with their cost, for the merge)
-  int64_t rows_total = 0;
-  for (const int k : keys) rows_total += ko1[k + 1] - ko1[k];
-  std::vector<int4> wide;
-  std::vector<std::pair<float, int4>> by_shape[UNG_SHAPES];
+  std::vector<PlannedTile>& wide = lists.wide;
+  std::vector<PlannedTile>(&by_shape)[UNG_SHAPES] = lists.by_shape;
   std::vector<int4>* out = largest_first ? nullptr : &tl->tiles;  // plain schedule: key by key
-  if (out) {
-    out->reserve((size_t)(rows_total / UNG_T1 + 4 * keys.size()));
-  } else {
-    wide.reserve((size_t)(rows_total / UNG_T1 + keys.size()));
-    by_shape[UNG_NARROW16].reserve((size_t)(std::min<int64_t>(rows_total / 16, 8 * (int64_t)keys.size()) + 16));
-    by_shape[UNG_NARROW].reserve(keys.size());
-    by_shape[UNG_NARROW4].reserve(keys.size());
-    by_shape[UNG_NARROW2].reserve(keys.size());
-  }
   double cost_now[UNG_SHAPES] = {};  // tile costs of the current key's n2
   int32_t n2_now = 0;
   // cheapest cover of the last t < 16 rows of a key by narrow tiles (a tile
@@ -352,36 +358,39 @@ void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first
   int64_t cover_passes = -1;
   double rests_gain = 0;  // of the keys' rests as wide tiles, over narrow ones
   bool full_wide = false;
-  auto emit = [&](int k, int64_t first, int64_t rows, int shape) {
+  // a wide tile's cost for the current key: a pass's, by 32 rows, times its
+  // passes
+  auto wide_cost = [&](int64_t rows) { return tile_cost(c, UNG_WIDE, n2_now, rows); };
+  auto emit = [&](int k, int64_t first, int64_t rows, int shape, std::vector<PlannedTile>* lists_of_shape) {
     const int4 t = make_tile(k, (int)first, (int)rows, shape, 0, n2_now);
     if (out) out->push_back(t);
-    else if (shape == UNG_WIDE) wide.push_back(t);
-    else by_shape[shape].push_back({(float)cost_now[shape], t});
+    else if (shape == UNG_WIDE) wide.push_back({wide_cost(tensor ? rows : UNG_T1), t});
+    else lists_of_shape[shape].push_back({cost_now[shape], t});
   };
+  // Whether the rests that cost less as wide tiles become wide ones is known
+  // at the end (rests_gain): until then their narrow tiles wait in lists.rests.
+  const bool weigh_rests = tensor && mode == 0 && n_sms > 0 && largest_first;
   for (const int k : keys) {
     const int64_t n1 = ko1[k + 1] - ko1[k];
     const int64_t n2 = ko2[k + 1] - ko2[k];
     tl->pairs += n1 * n2;
     n2_now = (int32_t)n2;
-    for (int shape = UNG_NARROW; shape < UNG_SHAPES; shape++) cost_now[shape] = tile_cost(c, shape, n2);
+    const bool new_passes = round_up(n2, NARROW_PASS) != cover_passes;
+    if (new_passes)
+      for (int shape = UNG_NARROW; shape < UNG_SHAPES; shape++) cost_now[shape] = tile_cost(c, shape, n2);
     int64_t u = ko1[k];
     const int64_t end = ko1[k + 1];
     if (mode >= 2) {  // one narrow shape only
       const int shape = mode - 1, r = shape_rows(shape);
-      for (; u < end; u += r) emit(k, u, std::min<int64_t>(r, end - u), shape);
+      for (; u < end; u += r) emit(k, u, std::min<int64_t>(r, end - u), shape, by_shape);
       continue;
     }
     for (; end - u >= UNG_T1; u += UNG_T1) {
-      emit(k, u, UNG_T1, UNG_WIDE);
+      emit(k, u, UNG_T1, UNG_WIDE, nullptr);
       full_wide = true;
     }
     const int64_t rem = end - u;
-    if (rem <= 0) continue;
-    if (mode == 1) {
-      emit(k, u, rem, UNG_WIDE);
-      continue;
-    }
-    if (round_up(n2, NARROW_PASS) != cover_passes) {
+    if (new_passes && mode != 1) {
       cover_passes = round_up(n2, NARROW_PASS);
       best[0] = 0;
       pick[0] = 0;
@@ -394,6 +403,11 @@ void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first
         }
       }
     }
+    if (rem <= 0) continue;
+    if (mode == 1) {
+      emit(k, u, rem, UNG_WIDE, nullptr);
+      continue;
+    }
     // full tiles of 16 rows (or of 8 where those cost less per row), then
     // the cheapest cover of the rest; against one wide tile for it all
     const int bulk = cost_now[UNG_NARROW16] <= 2 * cost_now[UNG_NARROW] ? UNG_NARROW16 : UNG_NARROW;
@@ -401,24 +415,21 @@ void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first
     const int64_t full = rem / br;
     const int tail = (int)(rem % br);
     const double narrow_cost = (double)full * cost_now[bulk] + best[tail];
-    const double wide_cost = tile_cost(c, UNG_WIDE, n2, tensor ? rem : UNG_T1);
-    const double gain = (tensor ? NARROW_SHARE * narrow_cost : narrow_cost) - wide_cost;
-    if (!narrow_rests && gain >= 0) {
+    const double gain = (tensor ? NARROW_SHARE * narrow_cost : narrow_cost) - wide_cost(tensor ? rem : UNG_T1);
+    std::vector<PlannedTile>* to = by_shape;
+    if (gain >= 0) {
       rests_gain += gain;
-      emit(k, u, rem, UNG_WIDE);
-      continue;
+      emit(k, u, rem, UNG_WIDE, nullptr);
+      if (!weigh_rests || full_wide) continue;
+      to = lists.rests;
     }
-    for (int64_t i = 0; i < full; i++, u += br) emit(k, u, br, bulk);
+    for (int64_t i = 0; i < full; i++, u += br) emit(k, u, br, bulk, to);
     for (int t = tail; t > 0;) {
       const int shape = pick[t], r = std::min(shape_rows(shape), t);
-      emit(k, u, r, shape);
+      emit(k, u, r, shape, to);
       u += r;
       t -= r;
     }
-  }
-  if (tensor && mode == 0 && n_sms > 0 && rests_gain > 0 && !full_wide && rests_gain < WIDE_LAUNCH * n_sms) {
-    build_tiles_from(ko1, ko2, largest_first, tl, key_mask, shape_override, n_sms, tensor, listed, true);
-    return;
   }
   if (!largest_first) {
     for (const int4& t : tl->tiles) tl->n_wide += tile_shape(t) == UNG_WIDE;
@@ -426,32 +437,31 @@ void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first
   }
   // wide tiles (one launch), then the narrow ones (another), costliest first:
   // a merge of the per-shape narrow lists, each already in cost order
-  size_t total = wide.size();
-  for (const auto& v : by_shape) total += v.size();
-  tl->tiles.reserve(total);
-  tl->tiles.insert(tl->tiles.end(), wide.begin(), wide.end());
-  tl->n_wide = (int64_t)wide.size();
-  size_t at[UNG_SHAPES] = {};
-  for (;;) {
-    int pickd = -1;
-    float bestc = 0;
+  std::vector<PlannedTile>& narrow = lists.narrow;
+  auto merged = [](const std::vector<PlannedTile>& x, const std::vector<PlannedTile>& y,
+                   std::vector<PlannedTile>& to) {
+    to.resize(x.size() + y.size());
+    std::merge(x.begin(), x.end(), y.begin(), y.end(), to.begin(), costlier);
+  };
+  if (weigh_rests && !full_wide && rests_gain < WIDE_LAUNCH * n_sms) {
+    wide.clear();
     for (int shape = UNG_NARROW; shape < UNG_SHAPES; shape++) {
-      if (at[shape] >= by_shape[shape].size()) continue;
-      const float v = by_shape[shape][at[shape]].first;
-      if (pickd < 0 || v > bestc) pickd = shape, bestc = v;
+      if (lists.rests[shape].empty()) continue;
+      merged(by_shape[shape], lists.rests[shape], narrow);
+      by_shape[shape].swap(narrow);
     }
-    if (pickd < 0) break;
-    tl->tiles.push_back(by_shape[pickd][at[pickd]++].second);
   }
+  merged(by_shape[UNG_NARROW], by_shape[UNG_NARROW4], lists.half[0]);
+  merged(by_shape[UNG_NARROW2], by_shape[UNG_NARROW16], lists.half[1]);
+  merged(lists.half[0], lists.half[1], narrow);
   if (n_sms > 0) {
-    std::vector<int4> wide(tl->tiles.begin(), tl->tiles.begin() + tl->n_wide);
-    std::vector<int4> narrow(tl->tiles.begin() + tl->n_wide, tl->tiles.end());
-    split_long_tiles(c, wide, 0, (int64_t)wide.size(), (int64_t)n_sms, tensor);
-    split_long_tiles(c, narrow, 0, (int64_t)narrow.size(), (int64_t)UNG_NARROW_CTAS_PER_SM * n_sms, tensor);
-    tl->tiles.assign(wide.begin(), wide.end());
-    tl->n_wide = (int64_t)wide.size();
-    tl->tiles.insert(tl->tiles.end(), narrow.begin(), narrow.end());
+    split_long_tiles(c, wide, (int64_t)n_sms, tensor);
+    split_long_tiles(c, narrow, (int64_t)UNG_NARROW_CTAS_PER_SM * n_sms, tensor);
   }
+  tl->n_wide = (int64_t)wide.size();
+  tl->tiles.reserve(wide.size() + narrow.size());
+  for (const PlannedTile& t : wide) tl->tiles.push_back(t.tile);
+  for (const PlannedTile& t : narrow) tl->tiles.push_back(t.tile);
 }
 
 // Queues stage 2 over the tile list (its device copy is a.tiles): in the
