@@ -150,19 +150,15 @@ int num_sms() {
 // the plain wide kernel, which runs at an S1 below UNG_TC_MIN_S1, is charged
 // PLAIN_WIDE_SLOT for every row of the shape.
 constexpr int TC_FIXED_ROWS = 83;
-// A key's rest goes to the tensor kernel where that costs less than
-// NARROW_SHARE of the narrow tiles' charge (in a whole launch these come to
-// 0.85 - 0.9 of it: 187 x 70,000 proteins on narrow tiles alone are charged
-// 1.06 ms and take 0.93), and if no key fills a wide tile only when all rests
-// together save the launch and its ramps, WIDE_LAUNCH ns on every SM.
-// Measured, stage 2, rests by plain cost / by this rule / the better of that
-// and narrow tiles alone: 90 x 70,000 0.565 / 0.536 / 0.534 ms, 187 x 200,000
-// 2.575 / 2.48 / 2.48, 250 x 200,000 3.03 / 3.01 / 3.01, 400 x 70,000 1.459 /
-// 1.467 / 1.459 (narrow alone 1.77).
-constexpr double NARROW_SHARE = 0.87, WIDE_LAUNCH = 30000.0;
+// If no key fills a wide tile, the keys' rests go to the tensor kernel only when
+// together they save its launch and its ramps, WIDE_LAUNCH ns on every SM.
+// Measured, stage 2 by cost alone / by this rule: 90 x 20,000 proteins 0.224 /
+// 0.200 ms, 187 x 20,000 0.346 / 0.318, 90 x 70,000 0.500 / 0.475, 187 x 70,000
+// 0.873 / 0.845; from 250 x 70,000 on the same.
+constexpr double WIDE_LAUNCH = 30000.0;
 constexpr double PLAIN_WIDE_SLOT = 0.317, PLAIN_WIDE_TILE = 2960.0;
 std::mutex g_cost_mu;
-plast_tile_costs g_costs = {0.140, 3660.0, 0.479, 566.0, 0.616, 1101.0, 1.094, 1090.0, 12, 0, 0.416, 314.0};
+plast_tile_costs g_costs = {0.140, 3660.0, 0.369, 588.0, 0.409, 785.0, 0.566, 830.0, 12, 0, 0.352, 107.0};
 // 0: by cost; 1: wide only; 2, 3, 4, 5: narrow tiles of 8, 4, 2, 16 rows only
 std::atomic<int> g_shape{0};
 constexpr int64_t WIDE_PASS = 128;                         // bank-2 windows per CTA pass, wide tile
@@ -415,7 +411,7 @@ void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first
     const int64_t full = rem / br;
     const int tail = (int)(rem % br);
     const double narrow_cost = (double)full * cost_now[bulk] + best[tail];
-    const double gain = (tensor ? NARROW_SHARE * narrow_cost : narrow_cost) - wide_cost(tensor ? rem : UNG_T1);
+    const double gain = narrow_cost - wide_cost(tensor ? rem : UNG_T1);
     std::vector<PlannedTile>* to = by_shape;
     if (gain >= 0) {
       rests_gain += gain;
@@ -1520,12 +1516,19 @@ uint64_t splitmix(uint64_t& x) {
   return z ^ (z >> 31);
 }
 
-// n_seqs random proteins of `len` residues (codes 0..19 uniform), indexed
+// n_seqs random proteins of `len` residues, indexed: residues at the background
+// frequencies of Robinson and Robinson (1991), because the share of the pairs
+// that the tensor kernel's bound lets through depends on the composition
+// (uniform residues make its passes cost twice as much)
+constexpr int BACKGROUND[NAA] = {781, 512, 449, 537, 192, 426, 630, 738, 220, 514, 902, 574, 224, 386, 520, 712, 584, 133, 322, 644};  // in 10,000, codes 0..19
 int random_bank(int32_t n_seqs, int len, uint64_t seed, cudaStream_t st, plast_bank** out) {
   std::vector<int8_t> codes((size_t)n_seqs * len);
   std::vector<int64_t> off((size_t)n_seqs + 1);
   uint64_t x = seed;
-  for (auto& c : codes) c = (int8_t)(splitmix(x) % 20);
+  std::vector<int8_t> of(10000);
+  for (int c = 0, at = 0; c < NAA; c++)
+    for (int i = 0; i < BACKGROUND[c]; i++) of[at++] = (int8_t)c;
+  for (auto& c : codes) c = of[splitmix(x) % of.size()];
   for (int32_t i = 0; i <= n_seqs; i++) off[i] = (int64_t)i * len;
   int8_t* d_codes = nullptr;
   int64_t* d_off = nullptr;

@@ -32,12 +32,17 @@
 //      for ALU-pipe work, which has none; the rest are int8.
 //  * narrow: up to R = 16, 8, 4 or 2 rows.  Every lane scores its own bank-2
 //    window (32 per warp) against the R rows: the profile holds one word per
-//    (k, b) and 4 rows (R / 4 planes for R >= 8), or one halfword per (k, b)
-//    and 2 rows; the 22 entries of a cell lie in distinct banks, so 32 lanes
-//    with any residues read them in one wavefront.  16- and 8-row tiles take
-//    the lanes' windows through shared memory; 4- and 2-row tiles, which do too little
-//    arithmetic per cell to hide a shared byte load, keep each lane's window
-//    in registers.  Narrow tiles serve short lists (a small query bank
+//    (k, b) and 4 rows (R / 4 planes for R >= 8), or one word of two int16 per
+//    (k, b) and 2 rows; the 22 entries of a cell lie in distinct banks, so 32
+//    lanes with any residues read them in one wavefront.  Each lane keeps its
+//    window in registers and takes a cell's profile address from it with one
+//    four-way dot product (byte times four plus the profile's address), on the
+//    FMA pipe: with a byte extraction and an address of their own, or a shared
+//    byte load a cell, the ALU and the LSU were the bound (20 x 100,000
+//    proteins 0.26 ms where this takes 0.21, 60 x 100,000 0.54 and 0.46, 250 x
+//    100,000 in 16-row tiles 1.96 and 1.85, in 2-row tiles 2.67 and 2.19).
+//    Now issue (72 %), the LSU (74 %), the FMA pipe (60 %) and DRAM (62 %) are
+//    near balance.  Narrow tiles serve short lists (a small query bank
 //    against a large one, the remainder of a long list), where a wide tile
 //    would mostly score padding rows.
 // The host picks the shape per key from measured per-cell and per-tile costs.
@@ -91,18 +96,16 @@ struct Wide {
 };
 
 // narrow tiles (their own kernel)
-constexpr int NSTRIDE = 52;                                // staged window stride: 13 words, conflict-free bytes
 constexpr int NPLANE = WIN * NCODE * 4;                     // 4224: one plane of 4 rows
 constexpr int NR_MAX = 16;                                  // rows of the largest narrow tile
 constexpr int NPROF_BYTES = (NR_MAX / 4) * NPLANE;          // 16896
 constexpr int NROWS_BYTES = WIN * NR_MAX;                   // 768, cell-major
 constexpr int NT_THREADS = 512;                            // narrow kernel: 2 CTAs of 16 warps per SM
 constexpr int NT_WARPS = NT_THREADS / 32;
-constexpr int NSTAGE_BYTES = NT_WARPS * 32 * NSTRIDE;      // 26624: one window per lane
 constexpr int NWKEY_BYTES = NT_WARPS * WBUF * 8;           // 4096
 constexpr int NWVAL_BYTES = NT_WARPS * WBUF * 4;           // 2048
 static_assert(UNG_NARROW_PASS == NT_WARPS * 32, "narrow pass = one window per lane");
-static_assert(NPROF_BYTES % 16 == 0 && NROWS_BYTES % 16 == 0 && (32 * NSTRIDE) % 16 == 0, "alignment");
+static_assert(NPROF_BYTES % 16 == 0 && NROWS_BYTES % 16 == 0, "alignment");
 static_assert(Wide<UNG_MAX_N16>::SMEM <= 232448, "shared memory per CTA");
 
 // bytes 2h, 2h+1 of x, sign-extended into the two halves of an int16x2
@@ -192,61 +195,51 @@ __device__ __forceinline__ void wide_pairs(uint32_t row, const unsigned char* pl
   }
 }
 
-// The lane's 2 * NW narrow row scores of cell k against bank-2 residue b,
-// as NW int16x2 words.  NW >= 2: rows 4p .. 4p+3 the word at
-// plane + p * NPLANE + (k * NCODE + b) * 4, p < NW / 2; NW = 1: rows 0-1 the
-// halfword at plane + (k * NCODE + b) * 2.
-template <int NW>
-__device__ __forceinline__ void narrow_scores(const unsigned char* plane, int k, uint32_t b, uint32_t (&u)[NW]) {
+template <int OFF>
+__device__ __forceinline__ uint32_t lds_u32(uint32_t saddr) {
+  uint32_t v;
+  asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(v) : "r"(saddr), "n"(OFF));
+  return v;
+}
+
+// The lane's 2 * NW narrow row scores of plane K (a cell's, or a folded seed
+// plane's) against the residue in byte C of its window, as NW int16x2 words:
+// one four-way dot product makes the address, the profile's (shared) plus four
+// times the byte.  NW >= 2: rows 4p .. 4p+3 the word at p * NPLANE + (K * NCODE
+// + b) * 4, p < NW / 2; NW = 1: rows 0-1 a word of two int16.
+template <int K, int C, int NW>
+__device__ __forceinline__ void narrow_scores(const uint32_t (&win)[12], uint32_t prof, uint32_t (&u)[NW]) {
+  const uint32_t at = __dp4a(win[C >> 2], 4u << (8 * (C & 3)), prof);
   if constexpr (NW == 1) {
-    uint32_t h;
-    asm("ld.shared.u16 %0, [%1];"
-        : "=r"(h)
-        : "r"((uint32_t)__cvta_generic_to_shared(plane + (k * NCODE + b) * 2)));
-    u[0] = sext_pair(h, 0);
+    u[0] = lds_u32<K * NCODE * 4>(at);
   } else {
-    const unsigned char* e = plane + (k * NCODE + b) * 4;
-#pragma unroll
-    for (int p = 0; p < NW / 2; p++) {
-      const uint32_t x = *reinterpret_cast<const uint32_t*>(e + p * NPLANE);
-      u[2 * p] = sext_pair(x, 0);
-      u[2 * p + 1] = sext_pair(x, 1);
+    const uint32_t x = lds_u32<K * NCODE * 4>(at);
+    u[0] = sext_pair(x, 0);
+    u[1] = sext_pair(x, 1);
+    if constexpr (NW >= 4) {
+      const uint32_t y = lds_u32<NPLANE + K * NCODE * 4>(at);
+      u[2] = sext_pair(y, 0);
+      u[3] = sext_pair(y, 1);
+    }
+    if constexpr (NW == 8) {
+      const uint32_t y = lds_u32<2 * NPLANE + K * NCODE * 4>(at), z = lds_u32<3 * NPLANE + K * NCODE * 4>(at);
+      u[4] = sext_pair(y, 0);
+      u[5] = sext_pair(y, 1);
+      u[6] = sext_pair(z, 0);
+      u[7] = sext_pair(z, 1);
     }
   }
 }
 
+// Cells K and K+1 of the lane's window (cell k = byte k of win) against the
+// tile's rows, then the following pairs (K = 4, 6, .., 46).
 template <int K, int NW>
-__device__ __forceinline__ void narrow_pairs(uint32_t row, const unsigned char* plane, uint32_t (&s)[NW],
-                                             uint32_t (&m)[NW]) {
-  if constexpr (K < WIN) {
-    const uint32_t b0 = lds_u8<K>(row), b1 = lds_u8<K + 1>(row);
-    uint32_t u0[NW], u1[NW];
-    narrow_scores<NW>(plane, K, b0, u0);
-    narrow_scores<NW>(plane, K + 1, b1, u1);
-#pragma unroll
-    for (int w = 0; w < NW; w++) {
-      const uint32_t t0 = __vadd2(s[w], u0[w]);
-      s[w] = __vadd2(t0, u1[w]);
-      m[w] = __vimax3_s16x2(m[w], t0, s[w]);
-    }
-    if constexpr (K + 1 == RIGHT - 1) {
-#pragma unroll
-      for (int w = 0; w < NW; w++) s[w] = m[w];
-    }
-    narrow_pairs<K + 2, NW>(row, plane, s, m);
-  }
-}
-
-// The same with the lane's window in registers (cell k = byte k of win).
-template <int K, int NW>
-__device__ __forceinline__ void narrow_pairs_reg(const uint32_t (&win)[12], const unsigned char* plane,
+__device__ __forceinline__ void narrow_pairs(const uint32_t (&win)[12], uint32_t plane,
                                                  uint32_t (&s)[NW], uint32_t (&m)[NW]) {
   if constexpr (K < WIN) {
-    const uint32_t b0 = (win[K >> 2] >> (8 * (K & 3))) & 0xffu;
-    const uint32_t b1 = (win[(K + 1) >> 2] >> (8 * ((K + 1) & 3))) & 0xffu;
     uint32_t u0[NW], u1[NW];
-    narrow_scores<NW>(plane, K, b0, u0);
-    narrow_scores<NW>(plane, K + 1, b1, u1);
+    narrow_scores<K, K, NW>(win, plane, u0);
+    narrow_scores<K + 1, K + 1, NW>(win, plane, u1);
 #pragma unroll
     for (int w = 0; w < NW; w++) {
       const uint32_t t0 = __vadd2(s[w], u0[w]);
@@ -257,7 +250,7 @@ __device__ __forceinline__ void narrow_pairs_reg(const uint32_t (&win)[12], cons
 #pragma unroll
       for (int w = 0; w < NW; w++) s[w] = m[w];
     }
-    narrow_pairs_reg<K + 2, NW>(win, plane, s, m);
+    narrow_pairs<K + 2, NW>(win, plane, s, m);
   }
 }
 
@@ -435,13 +428,12 @@ __device__ __forceinline__ uint32_t pack4(uint32_t src, const int8_t* tab, int b
 
 // A narrow tile of 2 * NW rows: rows cell-major (nrows[k][r], stride
 // NR_MAX), the profile (NW >= 2: planes nprof[p][k][b] of rows 4p .. 4p+3,
-// p < NW / 2; NW = 1: halfwords of rows 0-1; cells 0-3 folded into P1, M1,
+// p < NW / 2; NW = 1: words of two int16, rows 0-1; cells 0-3 folded into P1, M1,
 // P2 as in the wide tiles), then every bank-2 window of the key against it,
 // one per lane.
 template <int NW>
 __device__ __forceinline__ void narrow_tile(const UngArgs& a, int rows, int64_t u0, int64_t v0, int64_t v1,
-                                            uint8_t* nrows, unsigned char* nprof, const int8_t* tab,
-                                            unsigned char* my_nstage, uint32_t my_nrow, uint32_t s1x2,
+                                            uint8_t* nrows, unsigned char* nprof, const int8_t* tab, uint32_t s1x2,
                                             uint64_t* my_wk, uint32_t* my_wv, int& wcnt) {
   constexpr int NQ = NW >= 2 ? NW / 2 : 1;  // 4-row words per (cell, residue)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -484,7 +476,7 @@ __device__ __forceinline__ void narrow_tile(const UngArgs& a, int rows, int64_t 
       }
     }
     if constexpr (NW == 1) {
-      *reinterpret_cast<uint16_t*>(nprof + e * 2) = (uint16_t)(w[0] & 0xffffu);
+      *reinterpret_cast<uint32_t*>(nprof + e * 4) = sext_pair(w[0], 0);
     } else {
 #pragma unroll
       for (int q = 0; q < NQ; q++) *reinterpret_cast<uint32_t*>(nprof + q * NPLANE + e * 4) = w[q];
@@ -492,96 +484,43 @@ __device__ __forceinline__ void narrow_tile(const UngArgs& a, int rows, int64_t 
   }
   __syncthreads();
 
-  // window indexes relative to the key's first (32-bit arithmetic)
-  if constexpr (NW <= 2) {
-    // 2 or 4 rows: few operations per cell, so the lane's own window stays in
-    // registers (three 16-byte loads, one iteration ahead) and each cell's
-    // residue is a byte of it, not a shared-memory load
-    const int n2 = (int)(v1 - v0);
-    const uint4* src = reinterpret_cast<const uint4*>(a.nb2 + v0 * WIN);
-    uint4 cur[3];
-    {
-      const int v = warp * 32 + lane;
-#pragma unroll
-      for (int j = 0; j < 3; j++) cur[j] = v < n2 ? __ldg(src + (int64_t)v * 3 + j) : sent16;
-    }
-    for (int vb = warp * 32; vb < n2; vb += NT_WARPS * 32) {
-      const bool vok = vb + lane < n2;
-      uint4 nxt[3];
-      {
-        const int vn = vb + NT_WARPS * 32 + lane;
-#pragma unroll
-        for (int j = 0; j < 3; j++) nxt[j] = vn < n2 ? __ldg(src + (int64_t)vn * 3 + j) : sent16;
-      }
-      const uint32_t win[12] = {cur[0].x, cur[0].y, cur[0].z, cur[0].w, cur[1].x, cur[1].y,
-                                cur[1].z, cur[1].w, cur[2].x, cur[2].y, cur[2].z, cur[2].w};
-      uint32_t s[NW], m[NW];
-      {  // cells 0-3 from the folded seed planes
-        const uint32_t bs1 = (win[0] >> 8) & 0xffu, bs2 = (win[0] >> 16) & 0xffu;
-        uint32_t up[NW], uq[NW];
-        narrow_scores<NW>(nprof, 0, bs1, up);
-        narrow_scores<NW>(nprof, 2, bs2, uq);
-#pragma unroll
-        for (int w = 0; w < NW; w++) s[w] = __vadd2(up[w], uq[w]);
-        narrow_scores<NW>(nprof, 1, bs1, up);
-#pragma unroll
-        for (int w = 0; w < NW; w++) m[w] = __vmaxs2(up[w], s[w]);
-      }
-      narrow_pairs_reg<FIRST_CELL, NW>(win, nprof, s, m);
-      emit_hits<NW>(m, vok, rows, u0, v0 + vb + lane, a, s1x2, lane, my_wk, my_wv, wcnt);
-#pragma unroll
-      for (int j = 0; j < 3; j++) cur[j] = nxt[j];
-    }
-    return;
-  }
-  // the warp's 32 windows are 96 consecutive 16-byte items; lane l moves
-  // items l, l + 32, l + 64 (window q / 3, part q % 3), one iteration ahead
-  int nw[3], np[3];
-#pragma unroll
-  for (int j = 0; j < 3; j++) {
-    nw[j] = (lane + 32 * j) / 3;
-    np[j] = (lane + 32 * j) % 3;
-  }
-  // window indexes relative to the key's first (32-bit arithmetic)
+  // The lane's own window stays in registers (three 16-byte loads, one
+  // iteration ahead): a cell's residue is a byte of it, never loaded again.
+  // Window indexes are relative to the key's first (32-bit arithmetic).
   const int n2 = (int)(v1 - v0);
+  const uint32_t prof_s = (uint32_t)__cvta_generic_to_shared(nprof);
   const uint4* src = reinterpret_cast<const uint4*>(a.nb2 + v0 * WIN);
-  uint4 pre[3];
+  uint4 cur[3];
+  {
+    const int v = warp * 32 + lane;
 #pragma unroll
-  for (int j = 0; j < 3; j++) {
-    const int v = warp * 32 + nw[j];
-    pre[j] = v < n2 ? __ldg(src + (int64_t)v * 3 + np[j]) : sent16;
+    for (int j = 0; j < 3; j++) cur[j] = v < n2 ? __ldg(src + (int64_t)v * 3 + j) : sent16;
   }
   for (int vb = warp * 32; vb < n2; vb += NT_WARPS * 32) {
     const bool vok = vb + lane < n2;
-    __syncwarp();
+    uint4 nxt[3];
+    {
+      const int vn = vb + NT_WARPS * 32 + lane;
 #pragma unroll
-    for (int j = 0; j < 3; j++) {
-      uint32_t* d = reinterpret_cast<uint32_t*>(my_nstage + nw[j] * NSTRIDE + np[j] * 16);
-      d[0] = pre[j].x;
-      d[1] = pre[j].y;
-      d[2] = pre[j].z;
-      d[3] = pre[j].w;
+      for (int j = 0; j < 3; j++) nxt[j] = vn < n2 ? __ldg(src + (int64_t)vn * 3 + j) : sent16;
     }
-    __syncwarp();
-#pragma unroll
-    for (int j = 0; j < 3; j++) {
-      const int vn = vb + NT_WARPS * 32 + nw[j];
-      pre[j] = vn < n2 ? __ldg(src + (int64_t)vn * 3 + np[j]) : sent16;
-    }
+    const uint32_t win[12] = {cur[0].x, cur[0].y, cur[0].z, cur[0].w, cur[1].x, cur[1].y,
+                              cur[1].z, cur[1].w, cur[2].x, cur[2].y, cur[2].z, cur[2].w};
     uint32_t s[NW], m[NW];
     {  // cells 0-3 from the folded seed planes
-      const uint32_t bs1 = lds_u8<1>(my_nrow), bs2 = lds_u8<2>(my_nrow);
       uint32_t up[NW], uq[NW];
-      narrow_scores<NW>(nprof, 0, bs1, up);
-      narrow_scores<NW>(nprof, 2, bs2, uq);
+      narrow_scores<0, 1, NW>(win, prof_s, up);
+      narrow_scores<2, 2, NW>(win, prof_s, uq);
 #pragma unroll
       for (int w = 0; w < NW; w++) s[w] = __vadd2(up[w], uq[w]);
-      narrow_scores<NW>(nprof, 1, bs1, up);
+      narrow_scores<1, 1, NW>(win, prof_s, up);
 #pragma unroll
       for (int w = 0; w < NW; w++) m[w] = __vmaxs2(up[w], s[w]);
     }
-    narrow_pairs<FIRST_CELL, NW>(my_nrow, nprof, s, m);
+    narrow_pairs<FIRST_CELL, NW>(win, prof_s, s, m);
     emit_hits<NW>(m, vok, rows, u0, v0 + vb + lane, a, s1x2, lane, my_wk, my_wv, wcnt);
+#pragma unroll
+    for (int j = 0; j < 3; j++) cur[j] = nxt[j];
   }
 }
 
@@ -746,8 +685,8 @@ __global__ void __launch_bounds__(UNG_THREADS, 1) k_ungapped(UngArgs a) {
 // wide kernel's registers and schedule are its own; two CTAs of 512 threads
 // per SM, so that one CTA's tile changes (profile build, barriers) overlap
 // the other's scoring.
-constexpr int NARROW_SMEM = TAB_BYTES + NROWS_BYTES + NPROF_BYTES + NSTAGE_BYTES + NWKEY_BYTES + NWVAL_BYTES + 2 * 48;
-static_assert((TAB_BYTES + NROWS_BYTES + NPROF_BYTES + NSTAGE_BYTES) % 16 == 0, "alignment");
+constexpr int NARROW_SMEM = TAB_BYTES + NROWS_BYTES + NPROF_BYTES + NWKEY_BYTES + NWVAL_BYTES + 2 * 48;
+static_assert((TAB_BYTES + NROWS_BYTES + NPROF_BYTES) % 16 == 0, "alignment");
 static_assert(2 * NARROW_SMEM <= 228 * 1024, "two narrow CTAs per SM");
 
 __global__ void __launch_bounds__(NT_THREADS, 2) k_ungapped_narrow(UngArgs a) {
@@ -755,16 +694,14 @@ __global__ void __launch_bounds__(NT_THREADS, 2) k_ungapped_narrow(UngArgs a) {
   int8_t* tab = reinterpret_cast<int8_t*>(smem);
   uint8_t* nrows = smem + TAB_BYTES;
   unsigned char* nprof = smem + TAB_BYTES + NROWS_BYTES;
-  unsigned char* nstage = smem + TAB_BYTES + NROWS_BYTES + NPROF_BYTES;
-  uint64_t* wkey = reinterpret_cast<uint64_t*>(nstage + NSTAGE_BYTES);
-  uint32_t* wval = reinterpret_cast<uint32_t*>(nstage + NSTAGE_BYTES + NWKEY_BYTES);
-  TileSlot* slots = reinterpret_cast<TileSlot*>(nstage + NSTAGE_BYTES + NWKEY_BYTES + NWVAL_BYTES);
+  unsigned char* bufs = smem + TAB_BYTES + NROWS_BYTES + NPROF_BYTES;
+  uint64_t* wkey = reinterpret_cast<uint64_t*>(bufs);
+  uint32_t* wval = reinterpret_cast<uint32_t*>(bufs + NWKEY_BYTES);
+  TileSlot* slots = reinterpret_cast<TileSlot*>(bufs + NWKEY_BYTES + NWVAL_BYTES);
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   uint64_t* my_wk = wkey + warp * WBUF;
   uint32_t* my_wv = wval + warp * WBUF;
-  unsigned char* my_nstage = nstage + warp * 32 * NSTRIDE;
-  const uint32_t my_nrow = (uint32_t)__cvta_generic_to_shared(my_nstage + lane * NSTRIDE);
   int wcnt = 0;
 
   for (int i = tid; i < NCODE * NCODE; i += NT_THREADS) tab[i] = c_score[i];
@@ -780,13 +717,13 @@ __global__ void __launch_bounds__(NT_THREADS, 2) k_ungapped_narrow(UngArgs a) {
     const int64_t u0 = (int64_t)(uint32_t)tile.y;
     const int shape = tile_shape(tile);
     if (shape == UNG_NARROW16)
-      narrow_tile<8>(a, rows, u0, v0, v1, nrows, nprof, tab, my_nstage, my_nrow, s1x2, my_wk, my_wv, wcnt);
+      narrow_tile<8>(a, rows, u0, v0, v1, nrows, nprof, tab, s1x2, my_wk, my_wv, wcnt);
     else if (shape == UNG_NARROW)
-      narrow_tile<4>(a, rows, u0, v0, v1, nrows, nprof, tab, my_nstage, my_nrow, s1x2, my_wk, my_wv, wcnt);
+      narrow_tile<4>(a, rows, u0, v0, v1, nrows, nprof, tab, s1x2, my_wk, my_wv, wcnt);
     else if (shape == UNG_NARROW4)
-      narrow_tile<2>(a, rows, u0, v0, v1, nrows, nprof, tab, my_nstage, my_nrow, s1x2, my_wk, my_wv, wcnt);
+      narrow_tile<2>(a, rows, u0, v0, v1, nrows, nprof, tab, s1x2, my_wk, my_wv, wcnt);
     else
-      narrow_tile<1>(a, rows, u0, v0, v1, nrows, nprof, tab, my_nstage, my_nrow, s1x2, my_wk, my_wv, wcnt);
+      narrow_tile<1>(a, rows, u0, v0, v1, nrows, nprof, tab, s1x2, my_wk, my_wv, wcnt);
     __syncthreads();  // the next tile rebuilds the profile
   }
   if (wcnt > 0) {
