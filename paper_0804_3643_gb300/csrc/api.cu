@@ -158,7 +158,7 @@ constexpr int TC_FIXED_ROWS = 83;
 constexpr double WIDE_LAUNCH = 30000.0;
 constexpr double PLAIN_WIDE_SLOT = 0.317, PLAIN_WIDE_TILE = 2960.0;
 std::mutex g_cost_mu;
-plast_tile_costs g_costs = {0.140, 3660.0, 0.369, 588.0, 0.409, 785.0, 0.566, 830.0, 12, 0, 0.352, 107.0};
+plast_tile_costs g_costs = {0.140, 3660.0, 0.352, 729.0, 0.409, 783.0, 0.565, 831.0, 12, 0, 0.323, 383.0};
 // 0: by cost; 1: wide only; 2, 3, 4, 5: narrow tiles of 8, 4, 2, 16 rows only
 std::atomic<int> g_shape{0};
 constexpr int64_t WIDE_PASS = 128;                         // bank-2 windows per CTA pass, wide tile

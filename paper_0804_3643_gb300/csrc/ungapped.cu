@@ -40,7 +40,7 @@
 //    FMA pipe: with a byte extraction and an address of their own, or a shared
 //    byte load a cell, the ALU and the LSU were the bound (20 x 100,000
 //    proteins 0.26 ms where this takes 0.21, 60 x 100,000 0.54 and 0.46, 250 x
-//    100,000 in 16-row tiles 1.96 and 1.85, in 2-row tiles 2.67 and 2.19).
+//    100,000 in 16-row tiles 1.96 and 1.72, in 2-row tiles 2.67 and 2.19).
 //    Now issue (72 %), the LSU (74 %), the FMA pipe (60 %) and DRAM (62 %) are
 //    near balance.  Narrow tiles serve short lists (a small query bank
 //    against a large one, the remainder of a long list), where a wide tile
@@ -96,9 +96,9 @@ struct Wide {
 };
 
 // narrow tiles (their own kernel)
-constexpr int NPLANE = WIN * NCODE * 4;                     // 4224: one plane of 4 rows
+constexpr int NPLANE = WIN * NCODE * 4;                     // 4224: one plane of 4 int8 or 2 int16 rows
 constexpr int NR_MAX = 16;                                  // rows of the largest narrow tile
-constexpr int NPROF_BYTES = (NR_MAX / 4) * NPLANE;          // 16896
+constexpr int NPROF_BYTES = (NR_MAX / 2) * NPLANE;          // 33792
 constexpr int NROWS_BYTES = WIN * NR_MAX;                   // 768, cell-major
 constexpr int NT_THREADS = 512;                            // narrow kernel: 2 CTAs of 16 warps per SM
 constexpr int NT_WARPS = NT_THREADS / 32;
@@ -202,16 +202,38 @@ __device__ __forceinline__ uint32_t lds_u32(uint32_t saddr) {
   return v;
 }
 
+// Cells whose scores a tile of 16 or 8 rows holds as int16: twice the loads, no
+// sign extension, so every other cell's share balances the LSU and the ALU
+// (250 x 100,000 proteins in 16-row tiles 1.72 ms, none 1.85, every third 1.75,
+// two of three 1.73; in 8-row tiles 1.55, 1.67, 1.57, -; 4-row tiles gain
+// nothing).
+template <int NW>
+__host__ __device__ constexpr bool narrow16(int k) {
+  return NW >= 4 && k >= FIRST_CELL && k % 2 == 0;
+}
+
 // The lane's 2 * NW narrow row scores of plane K (a cell's, or a folded seed
 // plane's) against the residue in byte C of its window, as NW int16x2 words:
 // one four-way dot product makes the address, the profile's (shared) plus four
 // times the byte.  NW >= 2: rows 4p .. 4p+3 the word at p * NPLANE + (K * NCODE
-// + b) * 4, p < NW / 2; NW = 1: rows 0-1 a word of two int16.
+// + b) * 4, p < NW / 2, or, as int16, rows 2w, 2w+1 the word at w * NPLANE +
+// the same, w < NW; NW = 1: rows 0-1 a word of two int16.
 template <int K, int C, int NW>
 __device__ __forceinline__ void narrow_scores(const uint32_t (&win)[12], uint32_t prof, uint32_t (&u)[NW]) {
   const uint32_t at = __dp4a(win[C >> 2], 4u << (8 * (C & 3)), prof);
   if constexpr (NW == 1) {
     u[0] = lds_u32<K * NCODE * 4>(at);
+  } else if constexpr (narrow16<NW>(K)) {
+    u[0] = lds_u32<K * NCODE * 4>(at);
+    u[1] = lds_u32<NPLANE + K * NCODE * 4>(at);
+    u[2] = lds_u32<2 * NPLANE + K * NCODE * 4>(at);
+    u[3] = lds_u32<3 * NPLANE + K * NCODE * 4>(at);
+    if constexpr (NW == 8) {
+      u[4] = lds_u32<4 * NPLANE + K * NCODE * 4>(at);
+      u[5] = lds_u32<5 * NPLANE + K * NCODE * 4>(at);
+      u[6] = lds_u32<6 * NPLANE + K * NCODE * 4>(at);
+      u[7] = lds_u32<7 * NPLANE + K * NCODE * 4>(at);
+    }
   } else {
     const uint32_t x = lds_u32<K * NCODE * 4>(at);
     u[0] = sext_pair(x, 0);
@@ -477,6 +499,12 @@ __device__ __forceinline__ void narrow_tile(const UngArgs& a, int rows, int64_t 
     }
     if constexpr (NW == 1) {
       *reinterpret_cast<uint32_t*>(nprof + e * 4) = sext_pair(w[0], 0);
+    } else if (narrow16<NW>(k)) {
+#pragma unroll
+      for (int q = 0; q < NQ; q++) {
+        *reinterpret_cast<uint32_t*>(nprof + 2 * q * NPLANE + e * 4) = sext_pair(w[q], 0);
+        *reinterpret_cast<uint32_t*>(nprof + (2 * q + 1) * NPLANE + e * 4) = sext_pair(w[q], 1);
+      }
     } else {
 #pragma unroll
       for (int q = 0; q < NQ; q++) *reinterpret_cast<uint32_t*>(nprof + q * NPLANE + e * 4) = w[q];
