@@ -787,21 +787,20 @@ int plast_index_bank(const int8_t* codes, const int64_t* seq_off, int32_t n_seqs
   int rc;
   {
     Scratch sc(st);
-    int* d_bad;
     int64_t* d_seq_off;
-    if ((rc = ck(sc.get(&d_bad, 1)))) return fail(rc);
-    if ((rc = ck(cudaMemsetAsync(d_bad, 0, sizeof(int), st)))) return fail(rc);
     if ((rc = ck(dev_alloc_async((void**)&b->pad_alloc, (size_t)(n_pad + 2 * PAD_SLACK), st)))) return fail(rc);
     b->pad = b->pad_alloc + PAD_SLACK;
     if ((rc = ck(cudaMemsetAsync(b->pad_alloc, SENTINEL, (size_t)(n_pad + 2 * PAD_SLACK), st)))) return fail(rc);
     if ((rc = ck(dev_alloc_async((void**)&b->pad_off, ((size_t)n_seqs + 1) * sizeof(int64_t), st)))) return fail(rc);
-    if ((rc = ck(dev_alloc_async((void**)&b->key_off, (NKEYS + 1) * sizeof(int64_t), st)))) return fail(rc);
+    // the offsets, and behind them the flag of a code out of range: one copy
+    if ((rc = ck(dev_alloc_async((void**)&b->key_off, (NKEYS + 2) * sizeof(int64_t), st)))) return fail(rc);
+    int* d_bad = reinterpret_cast<int*>(b->key_off + NKEYS + 1);
+    if ((rc = ck(cudaMemsetAsync(d_bad, 0, sizeof(int64_t), st)))) return fail(rc);
     if ((rc = ck(cudaMemcpyAsync(b->pad_off, b->h_pad_off.data(), b->h_pad_off.size() * sizeof(int64_t),
                                  cudaMemcpyHostToDevice, st))))
       return fail(rc);
     if ((rc = ck(dev_alloc_async((void**)&b->blk_seq, ((size_t)(n_pad / SEQ_BLK) + 1) * sizeof(int32_t), st))))
       return fail(rc);
-    if ((rc = ck(launch_block_seq(b->pad_off, n_seqs, n_pad, b->blk_seq, st)))) return fail(rc);
     if ((rc = ck(sc.get(&d_seq_off, (size_t)n_seqs + 1)))) return fail(rc);
     if ((rc = ck(cudaMemcpyAsync(d_seq_off, seq_off, ((size_t)n_seqs + 1) * sizeof(int64_t),
                                  cudaMemcpyDeviceToDevice, st))))
@@ -825,22 +824,22 @@ int plast_index_bank(const int8_t* codes, const int64_t* seq_off, int32_t n_seqs
     const size_t room = (size_t)std::max<int64_t>(n_res, 1);  // a word per residue at most
     if ((rc = ck(sc.get(&by_pos, room)))) return fail(rc);
     if ((rc = ck(sc.get(&by_lo, room)))) return fail(rc);
-    if ((rc = ck(launch_index_split(b->pad, n_pad, shape, d_off, by_pos, by_lo, st)))) return fail(rc);
-    int h_bad = 0;
-    b->h_key_off.resize(NKEYS + 1);
-    if ((rc = ck(cudaMemcpyAsync(b->h_key_off.data(), b->key_off, (NKEYS + 1) * sizeof(int64_t),
+    b->h_key_off.resize(NKEYS + 2);
+    if ((rc = ck(cudaMemcpyAsync(b->h_key_off.data(), b->key_off, (NKEYS + 2) * sizeof(int64_t),
                                  cudaMemcpyDeviceToHost, st))))
       return fail(rc);
-    if ((rc = ck(cudaMemcpyAsync(&h_bad, d_bad, sizeof(int), cudaMemcpyDeviceToHost, st)))) return fail(rc);
     if ((rc = ck(cudaStreamSynchronize(st)))) return fail(rc);
-    if (h_bad) return fail(PLAST_E_INVALID);
+    if (b->h_key_off[NKEYS + 1]) return fail(PLAST_E_INVALID);
+    b->h_key_off.resize(NKEYS + 1);
     const int64_t n_idx = b->n_idx = b->h_key_off[NKEYS];
     if ((rc = ck(dev_alloc_async((void**)&b->pos, (size_t)std::max<int64_t>(n_idx, 1) * sizeof(uint32_t), st))))
       return fail(rc);
-    // the lists are laid out while the caller goes on (later calls wait on
-    // b->ready)
     if ((rc = ck(dev_alloc_async((void**)&b->nb, (size_t)std::max<int64_t>(n_idx, 1) * WIN, st)))) return fail(rc);
+    // the lists are laid out while the caller goes on (later calls wait on
+    // b->ready); with every allocation made, nothing is freed under them
+    if ((rc = ck(launch_index_split(b->pad, n_pad, shape, d_off, by_pos, by_lo, st)))) return fail(rc);
     if ((rc = ck(launch_index_fill(b->pad, shape, d_off, by_pos, by_lo, b->pos, b->nb, st)))) return fail(rc);
+    if ((rc = ck(launch_block_seq(b->pad_off, n_seqs, n_pad, b->blk_seq, st)))) return fail(rc);
     if ((rc = ck(cudaEventCreateWithFlags(&b->ready, cudaEventDisableTiming)))) return fail(rc);
     if ((rc = ck(cudaEventRecord(b->ready, st)))) return fail(rc);
   }

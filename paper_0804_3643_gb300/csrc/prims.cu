@@ -82,12 +82,15 @@ cudaError_t upload_tables_once() {
 }
 
 // ---------------------------------------------------------------------------
-// Exclusive scan, int32 in -> int64 out, in three passes over tiles of
-// SCAN_TILE elements: tile sums, a one-CTA scan of the sums, tile scans.
+// Exclusive scan, int32 in -> int64 out, over tiles of SCAN_TILE elements: tile
+// sums, a one-CTA scan of the sums, tile scans.  Up to SCAN_FEW_TILES tiles (two
+// million elements, 8 KB of sums for the last CTA to read) the second launch,
+// 2 to 3 us of a few microseconds' work, goes: the tile scans add up the sums.
 // ---------------------------------------------------------------------------
 constexpr int SCAN_THREADS = 256;
 constexpr int SCAN_ITEMS = 8;
 constexpr int SCAN_TILE = SCAN_THREADS * SCAN_ITEMS;
+constexpr int64_t SCAN_FEW_TILES = 1024;
 
 __device__ __forceinline__ int64_t block_exclusive_scan(int64_t v, int64_t* total) {
   __shared__ int64_t s_warp[SCAN_THREADS / 32];
@@ -149,8 +152,20 @@ __global__ void k_scan_sums(int64_t* sums, int64_t nt, int64_t* d_total) {
   if (threadIdx.x == 0 && d_total) *d_total = carry;
 }
 
-__global__ void k_scan_tiles(const int32_t* in, int64_t n, const int64_t* sums, int64_t* out, const int64_t* n_dev) {
+// FEW: the sums are the tiles' own, and each CTA adds up those before its tile.
+template <bool FEW>
+__global__ void k_scan_tiles(const int32_t* in, int64_t n, const int64_t* sums, int64_t* out, int64_t* d_total,
+                             const int64_t* n_dev) {
   n = count_of(n, n_dev);
+  int64_t before = 0;
+  if (FEW) {
+    int64_t x = 0;
+    for (int64_t i = threadIdx.x; i < blockIdx.x; i += SCAN_THREADS) x += sums[i];
+    block_exclusive_scan(x, &before);
+    if (threadIdx.x == 0 && d_total && blockIdx.x == gridDim.x - 1) *d_total = before + sums[blockIdx.x];
+  } else {
+    before = sums[blockIdx.x];
+  }
   // thread t owns the contiguous items [t*ITEMS, t*ITEMS + ITEMS) of the tile
   int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
   int32_t v[SCAN_ITEMS];
@@ -161,7 +176,7 @@ __global__ void k_scan_tiles(const int32_t* in, int64_t n, const int64_t* sums, 
     v[r] = i < n ? in[i] : 0;
     acc += v[r];
   }
-  int64_t ex = block_exclusive_scan(acc, nullptr) + sums[blockIdx.x];
+  int64_t ex = block_exclusive_scan(acc, nullptr) + before;
 #pragma unroll
   for (int r = 0; r < SCAN_ITEMS; r++) {
     int64_t i = base + r;
@@ -186,10 +201,15 @@ cudaError_t scan_exclusive(const int32_t* in, int64_t* out, int64_t n, int64_t* 
   int64_t* sums = (int64_t*)tmp;
   note_launch();
   k_scan_tile_sums<<<(unsigned)nt, SCAN_THREADS, 0, st>>>(in, n, sums, n_dev);
+  if (nt <= SCAN_FEW_TILES) {
+    note_launch();
+    k_scan_tiles<true><<<(unsigned)nt, SCAN_THREADS, 0, st>>>(in, n, sums, out, d_total, n_dev);
+    return cudaGetLastError();
+  }
   note_launch();
   k_scan_sums<<<1, SCAN_THREADS, 0, st>>>(sums, nt, d_total);
   note_launch();
-  k_scan_tiles<<<(unsigned)nt, SCAN_THREADS, 0, st>>>(in, n, sums, out, n_dev);
+  k_scan_tiles<false><<<(unsigned)nt, SCAN_THREADS, 0, st>>>(in, n, sums, out, nullptr, n_dev);
   return cudaGetLastError();
 }
 
