@@ -52,8 +52,8 @@
 // does not stay in the instruction caches.
 //
 // What bounds it: instruction issue and the latency of the chains (a pass of
-// 128 windows x 128 rows takes 2.3 us on an SM: issue 63 %, shared memory
-// wavefronts 65 %, tensor pipe 33 %, ALU 48 %).  Stage 2 of 10,000 x 100,000
+// 128 windows x 128 rows takes 2.3 us on an SM: issue 66 %, shared memory
+// wavefronts 71 %, tensor pipe 33 %, ALU 48 %).  Stage 2 of 10,000 x 100,000
 // proteins (2.15e10 pairs): 20.6 ms, with the plain wide kernel 45.5 ms; of
 // 10,000 x 10,000: 3.1 ms against 4.5.  Measured on the way: fp32 maxima of
 // the accumulators (no base of 2^23) 33.8 ms; the one-hot steps by one warp

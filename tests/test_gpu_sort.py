@@ -66,3 +66,19 @@ def test_plan_with_room_to_spare(B, room):
         records, _ = plan.result()
         got = B.gapped_numpy(records)
         assert got.shape == want.shape and np.array_equal(got.view(np.uint8), want.view(np.uint8))
+
+
+@pytest.mark.parametrize("n", [1448, 1449])
+def test_scan_of_few_and_many_tiles(B, n):
+    # stage 3.1 of n * n given hits: 1,024 tiles of 2,048 flags and more
+    torch = pytest.importorskip("torch")
+    rng = np.random.default_rng(n)
+    (g1, o1), (g2, o2) = (both(B, one_word_bank(rng, n)) for _ in range(2))
+    key = oracle.seed_key([0, 5, 0, 0])
+    hits = oracle.ungapped(o1, o2, oracle.Params(s1=-30000), key_lo=key, key_hi=key + 1, threads=8)
+    assert len(hits) == n * n
+    prm = dict(s2=25)
+    want = oracle.small_gapped(o1, o2, hits, oracle.Params(**prm), threads=8)
+    assert n < len(want) < len(hits)
+    got = B.gapped_numpy(B.plast_small_gapped(g1, g2, B.hits_from_numpy(hits), B.plast_default_params(**prm)))
+    assert got.shape == want.shape and np.array_equal(got.view(np.uint8), want.view(np.uint8))
