@@ -1251,7 +1251,7 @@ int plast_translate6(const uint8_t* dna, const int64_t* contig_off, int32_t n_co
   int* d_bad;
   CK(sc.get(&d_bad, 1));
   CK(cudaMemsetAsync(d_bad, 0, sizeof(int), st));
-  CK(launch_check_codes((const int8_t*)dna, n_nt, 0, 3, d_bad, st));
+  CK(launch_check_codes((const int8_t*)dna, n_nt, 3, d_bad, st));
   int h_bad = 0;
   int rc = check_bad(d_bad, st, &h_bad);
   if (rc) return rc;

@@ -4,7 +4,7 @@
 
 namespace plast {
 
-cudaError_t launch_check_codes(const int8_t* codes, int64_t n, int lo, int hi, int* bad, cudaStream_t st);
+cudaError_t launch_check_codes(const int8_t* codes, int64_t n, int hi, int* bad, cudaStream_t st);
 // Codes into the sentinel-filled padded bank, checked against [0, hi].
 cudaError_t launch_build_pad(const int8_t* codes, const int64_t* seq_off, int32_t n_seqs, int64_t n_res, int hi,
                              int8_t* pad, int* bad, cudaStream_t st);
