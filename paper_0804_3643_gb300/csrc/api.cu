@@ -231,20 +231,20 @@ bool costlier(const PlannedTile& x, const PlannedTile& y) { return x.cost > y.co
 
 // The lists that a tile plan goes through, kept by the thread that plans: as
 // fresh vectors their page faults took half of a small search's planning.
-// Given back after a plan of more than a million tiles.
+// After a plan that grew them past a million tiles they are given back.
 struct PlanLists {
   std::vector<PlannedTile> wide, by_shape[UNG_SHAPES], rests[UNG_SHAPES], narrow, half[2], rest, pieces;
   std::vector<int> keys, sorted;
-  void clear() {
-    size_t held = 0;
+  size_t clear() {  // the tiles there is room for
+    size_t room = 0;
     auto each = [&](std::vector<PlannedTile>& v) {
-      held += v.capacity();
+      room += v.capacity();
       v.clear();
     };
     for (auto* v : {&wide, &narrow, &half[0], &half[1], &rest, &pieces}) each(*v);
     for (auto& v : by_shape) each(v);
     for (auto& v : rests) each(v);
-    if (held > 1 << 20) *this = PlanLists();
+    return room;
   }
 };
 PlanLists& plan_lists() {
@@ -458,6 +458,7 @@ void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first
   tl->tiles.reserve(wide.size() + narrow.size());
   for (const PlannedTile& t : wide) tl->tiles.push_back(t.tile);
   for (const PlannedTile& t : narrow) tl->tiles.push_back(t.tile);
+  if (lists.clear() > 1 << 20) lists = PlanLists();
 }
 
 // Queues stage 2 over the tile list (its device copy is a.tiles): in the
