@@ -171,7 +171,7 @@ int plast_translate6(const uint8_t* dna, const int64_t* contig_off, int32_t n_co
  *   params  may be NULL (defaults)
  *   *out    receives the new bank (host)
  * The inputs are consumed before the call returns; the caller may free them
- * then.  The last step (laying out the neighbourhoods) may still be running
+ * then.  The last steps (laying out the lists and windows) may still be running
  * on `stream` when the call returns: every later call that takes the bank
  * waits for it, on whatever stream it is given, and plast_bank_free waits
  * too, so the caller may go on to host work (another bank, planning) while
