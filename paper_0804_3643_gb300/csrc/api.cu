@@ -509,43 +509,58 @@ void build_tiles(const plast_bank* b1, const plast_bank* b2, bool largest_first,
 // thresholds that few pairs reach.
 bool stage2_on_tensor(const plast_params& prm) { return prm.s1 >= UNG_TC_MIN_S1; }
 
-// The survivor rate of the last stage 2 of each pair of banks, to size the
-// next one's survivor buffer.  The first guess, pairs / 128, holds for
-// ordinary protein banks (about 1 / 570 at S1 = 38), but keys with
-// low-complexity runs pass far more often, and an overflowing first run is
-// run again with the exact count; with the rate of the pair's last search
-// the buffer fits at once.  Sizing only: no result depends on it.
+// The survivor rate of the last stage 2 of each pair of banks at each threshold
+// over each choice of keys, to size the next one's survivor buffer.  The first guess, pairs /
+// 128, holds for ordinary protein banks (about 1 / 570 at S1 = 38), but keys
+// with low-complexity runs pass far more often, and an overflowing first run
+// is run again with the exact count; with the rate of the last like search the
+// buffer fits at once.  (A rate at another threshold or of other keys is no
+// measure: every pair of one key may pass where one in hundreds does of all.)
+// Sizing only: where the buffer of the rate cannot be had, the first guess
+// stands.
 struct RateHint {
   const plast_bank* b1;
   const plast_bank* b2;
+  int32_t s1;
+  uint64_t keys;  // hash of the key list, 0: every key
   double rate;
+  bool of(const plast_bank* x1, const plast_bank* x2, int32_t s, uint64_t k) const {
+    return b1 == x1 && b2 == x2 && s1 == s && keys == k;
+  }
 };
 std::mutex g_hint_mu;
 RateHint g_hints[32] = {};
 int g_hint_next = 0;
 
-double rate_hint(const plast_bank* b1, const plast_bank* b2) {
+uint64_t keys_hash(const std::vector<char>* mask) {
+  if (!mask) return 0;
+  uint64_t h = 0xcbf29ce484222325ull;  // FNV-1a
+  for (const char c : *mask) h = (h ^ (uint8_t)c) * 0x100000001b3ull;
+  return h | 1;
+}
+
+double rate_hint(const plast_bank* b1, const plast_bank* b2, int32_t s1, uint64_t keys) {
   std::lock_guard<std::mutex> lk(g_hint_mu);
   for (const RateHint& h : g_hints)
-    if (h.b1 == b1 && h.b2 == b2) return h.rate;
+    if (h.of(b1, b2, s1, keys)) return h.rate;
   return 0.0;
 }
 
-void set_rate_hint(const plast_bank* b1, const plast_bank* b2, double rate) {
+void set_rate_hint(const plast_bank* b1, const plast_bank* b2, int32_t s1, uint64_t keys, double rate) {
   std::lock_guard<std::mutex> lk(g_hint_mu);
   for (RateHint& h : g_hints)
-    if (h.b1 == b1 && h.b2 == b2) {
+    if (h.of(b1, b2, s1, keys)) {
       h.rate = rate;
       return;
     }
-  g_hints[g_hint_next] = RateHint{b1, b2, rate};
+  g_hints[g_hint_next] = RateHint{b1, b2, s1, keys, rate};
   g_hint_next = (g_hint_next + 1) % 32;
 }
 
 void forget_rate_hints(const plast_bank* b) {
   std::lock_guard<std::mutex> lk(g_hint_mu);
   for (RateHint& h : g_hints)
-    if (h.b1 == b || h.b2 == b) h = RateHint{nullptr, nullptr, 0.0};
+    if (h.b1 == b || h.b2 == b) h = RateHint{};
 }
 
 // Device state shared by the stage-2 calls: sorted survivor keys and values.
@@ -579,14 +594,25 @@ int run_ungapped(const plast_bank* b1, const plast_bank* b2, const plast_params&
   CK(sc.get(&d_count, 2));  // the survivors, then the kernels' error flag
   CK(cudaMemcpyAsync(d_tiles, tl.tiles.data(), nt * sizeof(int4), cudaMemcpyHostToDevice, st));
 
-  int64_t cap = tl.pairs / 128 + (1 << 20);
-  const double hint = rate_hint(b1, b2);
-  if (hint > 0.0) cap = std::max<int64_t>(cap, (int64_t)(hint * 1.1 * (double)tl.pairs) + (1 << 20));
+  const int64_t guess = tl.pairs / 128 + (1 << 20);
+  const uint64_t keys = keys_hash(key_mask);
+  const double hint = rate_hint(b1, b2, prm.s1, keys);
+  int64_t cap = std::max<int64_t>(guess, hint > 0.0 ? (int64_t)(hint * 1.1 * (double)tl.pairs) + (1 << 20) : 0);
   for (int attempt = 0; attempt < 2; attempt++) {
-    uint64_t *k0, *k1;
-    uint32_t *v0, *v1;
-    CK(sc.get(&k0, cap));
-    CK(sc.get(&v0, cap));
+    uint64_t *k0 = nullptr, *k1;
+    uint32_t *v0 = nullptr, *v1;
+    cudaError_t got = sc.get(&k0, cap);
+    if (got == cudaSuccess) got = sc.get(&v0, cap);
+    if (got == cudaErrorMemoryAllocation && attempt == 0 && cap > guess) {
+      // the rate asks for more than there is: the first guess, which an
+      // overflow turns into the exact count
+      cudaGetLastError();
+      if (k0) sc.release(k0);
+      cap = guess;
+      got = sc.get(&k0, cap);
+      if (got == cudaSuccess) got = sc.get(&v0, cap);
+    }
+    CK(got);
     CK(cudaMemsetAsync(d_counter, 0, 2 * sizeof(int32_t), st));
     CK(cudaMemsetAsync(d_count, 0, 2 * sizeof(unsigned long long), st));
     UngArgs a;
@@ -612,7 +638,7 @@ int run_ungapped(const plast_bank* b1, const plast_bank* b2, const plast_params&
     CK(cudaStreamSynchronize(st));
     if (h_count[1]) return PLAST_E_TIMEOUT;
     unsigned long long n = h_count[0];
-    if (tl.pairs > 0) set_rate_hint(b1, b2, (double)n / (double)tl.pairs);
+    if (tl.pairs > 0) set_rate_hint(b1, b2, prm.s1, keys, (double)n / (double)tl.pairs);
     if ((int64_t)n > cap) {
       sc.release(k0);
       sc.release(v0);
