@@ -364,6 +364,16 @@ void plast_plan_free(plast_plan* plan);
 int plast_set_alloc_limit(int64_t bytes);
 
 /*
+ * Fault injection for the failure paths (tests): from now on each wait between
+ * the warps of stage 2's tensor kernel gives up after `clocks` SM clocks, and
+ * the call (of a plan: plast_plan_result) reports PLAST_E_TIMEOUT; the device
+ * stays usable.  0, or more than the default: the default again, 4e9 (two seconds
+ * or so, a million times what a wait takes).  PLAST_E_INVALID if clocks < 0.  Applies to later launches in
+ * this process (a captured plan keeps the limit of its capture).
+ */
+int plast_set_wait_limit(int64_t clocks);
+
+/*
  * Scheduling of stage 2.  0 (default): one persistent launch, CTAs pull
  * profile tiles from a device work queue, largest first.  1: the plain
  * form, one launch per key.  Applies to later calls in this process.

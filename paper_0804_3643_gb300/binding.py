@@ -94,6 +94,8 @@ def lib() -> ctypes.CDLL:
         L.plast_strerror.restype = ctypes.c_char_p
         L.plast_set_alloc_limit.argtypes = [i64]
         L.plast_set_alloc_limit.restype = ctypes.c_int
+        L.plast_set_wait_limit.argtypes = [i64]
+        L.plast_set_wait_limit.restype = ctypes.c_int
         L.plast_set_schedule.argtypes = [ctypes.c_int]
         L.plast_set_schedule.restype = ctypes.c_int
         L.plast_translate6.argtypes = [P, P, i32, P, i64, P, P, pI64, P]
@@ -188,6 +190,14 @@ def plast_set_alloc_limit(nbytes: int) -> None:
     rc = lib().plast_set_alloc_limit(int(nbytes))
     if rc:
         raise PlastError("plast_set_alloc_limit", rc)
+
+
+def plast_set_wait_limit(clocks: int) -> None:
+    """Fault injection: the waits of stage 2's tensor kernel give up after
+    ``clocks`` SM clocks and the call raises with PLAST_E_TIMEOUT (0: the default)."""
+    rc = lib().plast_set_wait_limit(int(clocks))
+    if rc:
+        raise PlastError("plast_set_wait_limit", rc)
 
 
 def plast_set_schedule(mode: int) -> None:

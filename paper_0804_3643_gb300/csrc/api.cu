@@ -83,6 +83,9 @@ int rc_of(cudaError_t e) {
   return PLAST_E_CUDA;
 }
 
+// What the stage-2 kernels' error flag means to a caller.
+int rc_of_flag(unsigned long long flag) { return flag & UNG_ERR_TMEM ? PLAST_E_CUDA : PLAST_E_TIMEOUT; }
+
 #define CK(x)                              \
   do {                                     \
     cudaError_t e_ = (x);                  \
@@ -636,7 +639,7 @@ int run_ungapped(const plast_bank* b1, const plast_bank* b2, const plast_params&
     unsigned long long h_count[2] = {0, 0};
     CK(cudaMemcpyAsync(h_count, d_count, sizeof(h_count), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
-    if (h_count[1]) return PLAST_E_TIMEOUT;
+    if (h_count[1]) return rc_of_flag(h_count[1]);
     unsigned long long n = h_count[0];
     if (tl.pairs > 0) set_rate_hint(b1, b2, prm.s1, keys, (double)n / (double)tl.pairs);
     if ((int64_t)n > cap) {
@@ -739,6 +742,12 @@ long long plast_kernel_launches(void) { return plast::launch_total(); }
 int plast_set_alloc_limit(int64_t bytes) {
   if (bytes < 0) return PLAST_E_INVALID;
   g_alloc_limit.store(bytes);
+  return PLAST_OK;
+}
+
+int plast_set_wait_limit(int64_t clocks) {
+  if (clocks < 0) return PLAST_E_INVALID;
+  set_ungapped_wait_limit(clocks);
   return PLAST_OK;
 }
 
@@ -1515,7 +1524,7 @@ int plast_plan_result(const plast_plan* p, int64_t* n_records, int64_t* n_hits, 
   if (p->count_f) CK(cudaMemcpyAsync(&kept, p->count_f, sizeof(kept), cudaMemcpyDeviceToHost, st));
   CK(cudaMemcpyAsync(&recs, p->total, sizeof(recs), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
-  if (count[1]) return PLAST_E_TIMEOUT;
+  if (count[1]) return rc_of_flag(count[1]);
   const unsigned long long hits = count[0];
   if (n_hits) *n_hits = (int64_t)(p->count_f && hits <= (unsigned long long)p->max_hits ? kept : hits);
   if ((int64_t)hits > p->max_hits) {
@@ -1628,13 +1637,15 @@ int time_stage2(const plast_bank* b1, const plast_bank* b2, int shape, bool tens
   }
   std::vector<float> t;
   cudaError_t e = cudaSuccess;
-  for (int r = 0; r <= reps && e == cudaSuccess; r++) {
+  unsigned long long flag = 0;
+  for (int r = 0; r <= reps && e == cudaSuccess && flag == 0; r++) {
     e = cudaMemsetAsync(d_counter, 0, 2 * sizeof(int32_t), st);
     if (e == cudaSuccess) e = cudaMemsetAsync(d_count, 0, 2 * sizeof(unsigned long long), st);
     if (e == cudaSuccess) e = cudaEventRecord(e0, st);
     if (e == cudaSuccess) e = launch_tiles(tl, a, d_counter, true, st);
     if (e == cudaSuccess) e = cudaEventRecord(e1, st);
-    if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&flag, d_count + 1, sizeof(flag), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     float x = 0;
     if (e == cudaSuccess) e = cudaEventElapsedTime(&x, e0, e1);
     if (r > 0) t.push_back(x);  // run 0 warms up
@@ -1642,6 +1653,7 @@ int time_stage2(const plast_bank* b1, const plast_bank* b2, int shape, bool tens
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (e != cudaSuccess) return rc_of(e);
+  if (flag) return rc_of_flag(flag);  // an abandoned launch has no time
   std::sort(t.begin(), t.end());
   *ms = t[t.size() / 2];
   return PLAST_OK;
@@ -1762,7 +1774,7 @@ int plast_autotune(void* stream, plast_tile_costs* out) {
   for (int v = best_v % UNG_N16_VARIANTS + UNG_N16_VARIANTS; v < UNG_VARIANTS && rc == PLAST_OK;
        v += UNG_N16_VARIANTS)
     try_variant(v, false);
-  set_ungapped_variant(rc == PLAST_OK ? best_v : saved_variant);
+  set_ungapped_variant(best_v);
   double t_long;
   if (rc == PLAST_OK) rc = fit(1, true, &c.wide_slot, &c.wide_tile, &t_long);
   if (rc == PLAST_OK) rc = fit(2, false, &c.narrow_slot, &c.narrow_tile, &t_long);
@@ -1773,7 +1785,10 @@ int plast_autotune(void* stream, plast_tile_costs* out) {
   plast_bank_free(b1w);
   plast_bank_free(b2l);
   plast_bank_free(b2s);
-  if (rc != PLAST_OK) return rc;
+  if (rc != PLAST_OK) {
+    set_ungapped_variant(saved_variant);
+    return rc;
+  }
   rc = plast_set_tile_costs(&c);
   if (rc == PLAST_OK && out) *out = c;
   return rc;

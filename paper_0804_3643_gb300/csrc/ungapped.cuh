@@ -39,7 +39,7 @@ struct UngArgs {
   unsigned long long* out_count;
   int64_t cap;              // capacity of out_key / out_val
   int32_t sh;               // bits of a bank-2 padded position
-  int32_t* err;             // raised when a bounded wait of the tensor kernel ran out
+  int32_t* err;             // UNG_ERR_* bits of the tensor kernel
 };
 
 // Wide-tile variants of the stage-2 kernel: how many cells the profile holds
@@ -56,6 +56,12 @@ void set_ungapped_variant(int v);    // -1: the default
 cudaError_t launch_ungapped(const UngArgs& a, int grid, cudaStream_t st);
 cudaError_t launch_ungapped_narrow(const UngArgs& a, int grid, cudaStream_t st);
 cudaError_t launch_ungapped_mma(const UngArgs& a, int grid, cudaStream_t st);
+// The limit of each of the tensor kernel's waits, in SM clocks, and a shorter
+// one for later launches (0: the default again).
+constexpr uint32_t UNG_WAIT_CLOCKS = 4000000000u;
+void set_ungapped_wait_limit(int64_t clocks);
+constexpr int32_t UNG_ERR_WAIT = 1;  // a wait ran out
+constexpr int32_t UNG_ERR_TMEM = 2;  // tensor memory was not all the CTA's own
 constexpr int UNG_TC_PASS = 128;      // bank-2 windows the tensor kernel scores per pass
 // Lowest S1 whose wide tiles go to the tensor kernel: below it more pairs pass
 // the bound than their exact extension is worth (3,000 x 20,000 proteins, ms:

@@ -46,8 +46,9 @@
 //                      at a time exactly (one per lane), emit the hits
 //   4 MMA warps        issue a chain's MMAs each
 //   1 tile warp        fetches the tiles, ahead of the others
-// They meet at two mbarriers per segment and half.  Every wait has a limit; a
-// wait that runs out raises the launch's error flag and ends the CTA's work.
+// They meet at two mbarriers per segment and half.  Every wait has a limit
+// (struct Waits); a wait that runs out raises the launch's error flag and ends
+// the CTA's work.
 // The roles' loops are kept short: straight-line code of this many roles
 // does not stay in the instruction caches.
 //
@@ -158,9 +159,10 @@ constexpr int OFF_QUEUE = OFF_RING + EPI_WARPS * RING * 32 * 8;
 constexpr int OFF_HKEY = OFF_QUEUE + EXT_WARPS * QCAP * 8;
 constexpr int OFF_HVAL = OFF_HKEY + EXT_WARPS * HBUF * 8;
 constexpr int OFF_BAR = OFF_HVAL + EXT_WARPS * HBUF * 4;
-constexpr int OFF_MISC = OFF_BAR + (4 * NGROUP + 3) * 8;   // tensor memory address, abort flag, tiles fetched
+constexpr int OFF_WAITS = OFF_BAR + (4 * NGROUP + 3) * 8;  // abort flag and wait limit
+constexpr int OFF_MISC = OFF_WAITS + 8;                    // tensor memory address, tiles fetched
 // per epilogue warp: passes written, passes taken; per extend warp: tiles ended
-constexpr int OFF_RPOS = (OFF_MISC + 12 + 15) & ~15;
+constexpr int OFF_RPOS = (OFF_MISC + 8 + 15) & ~15;
 constexpr int RP_TAKEN = EPI_WARPS, RP_EXT = 2 * EPI_WARPS;
 constexpr int RP_WORDS = 2 * EPI_WARPS + EXT_WARPS;
 constexpr int OFF_SLOTS = (OFF_RPOS + RP_WORDS * 4 + 15) & ~15;
@@ -191,11 +193,26 @@ __device__ __forceinline__ void bar_init(uint32_t bar, uint32_t count) {
 __device__ __forceinline__ void bar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
-// Waits for the phase of the given parity, WAIT_CLOCKS at most (two seconds; a
-// pass takes microseconds); a wait that runs out raises *abort, and a raised
-// *abort ends every later wait.  (The votes keep the warp's lanes together:
-// loops that each lane leaves by itself cost more than the votes.)
-constexpr long long WAIT_CLOCKS = 4000000000ll;
+// A CTA's waits: each ends after `limit` clocks, UNG_WAIT_CLOCKS (two seconds; a
+// pass takes microseconds) unless a caller has set fewer; one that runs out
+// raises `abort`, and a raised `abort` ends every later wait.  The tile warp,
+// which waits for whole tiles, counts from the last pass that ended.  (Both
+// in one word of shared memory and 32-bit clocks: the limit in two registers
+// and 64 bits cost the stage 2 of ordinary banks 3 %.)
+struct Waits {
+  int abort;
+  uint32_t limit;
+};
+__device__ __forceinline__ uint32_t now() { return (uint32_t)clock(); }
+__device__ __forceinline__ bool over(Waits* waits, uint32_t t0) {  // (the whole warp)
+  int abort;
+  uint32_t limit;
+  asm volatile("ld.volatile.shared.v2.u32 {%0, %1}, [%2];" : "=r"(abort), "=r"(limit) : "r"(saddr(waits)) : "memory");
+  if (!__any_sync(0xffffffffu, abort || now() - t0 > limit)) return false;
+  *(volatile int*)&waits->abort = 1;
+  return true;
+}
+
 __device__ __forceinline__ bool bar_try(uint32_t bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -205,15 +222,14 @@ __device__ __forceinline__ bool bar_try(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok != 0u;
 }
-__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, volatile int* abort) {
+// Waits for the phase of the given parity.  (The votes keep the warp's lanes
+// together: loops that each lane leaves by itself cost more than the votes.)
+__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, Waits* waits) {
   if (__any_sync(0xffffffffu, bar_try(bar, parity))) return true;
-  const long long t0 = clock64();
+  const uint32_t t0 = now();
   for (;;) {
     if (__any_sync(0xffffffffu, bar_try(bar, parity))) return true;
-    if (__any_sync(0xffffffffu, *abort || clock64() - t0 > WAIT_CLOCKS)) {
-      *abort = 1;
-      return false;
-    }
+    if (over(waits, t0)) return false;
   }
 }
 
@@ -342,15 +358,12 @@ static_assert(sizeof(TileInfo) <= SLOT_INFO, "tile slot size");
 
 // Tile k of this CTA, once it has been fetched; false when there is
 // none or the launch has failed.
-__device__ __forceinline__ bool wait_tile(const unsigned char* smem, uint32_t k, TileInfo& t, volatile int* abort) {
-  volatile const uint32_t* fetched = reinterpret_cast<volatile const uint32_t*>(smem + OFF_MISC + 8);
+__device__ __forceinline__ bool wait_tile(const unsigned char* smem, uint32_t k, TileInfo& t, Waits* waits) {
+  volatile const uint32_t* fetched = reinterpret_cast<volatile const uint32_t*>(smem + OFF_MISC + 4);
   if (__any_sync(0xffffffffu, *fetched <= k)) {
-    const long long t0 = clock64();
+    const uint32_t t0 = now();
     while (__any_sync(0xffffffffu, *fetched <= k)) {
-      if (__any_sync(0xffffffffu, *abort || clock64() - t0 > WAIT_CLOCKS)) {
-        *abort = 1;
-        return false;
-      }
+      if (over(waits, t0)) return false;
       __nanosleep(64);
     }
   }
@@ -385,13 +398,13 @@ __device__ __forceinline__ void expand_step(int step, uint32_t win, uint32_t lut
 // One pass: one side of the lane's window to one-hot steps, segment by segment
 // as their last use has ended.
 __device__ __forceinline__ bool expand_pass(int side, uint32_t win, uint32_t lut, uint32_t tm, uint32_t bars,
-                                            uint32_t pass, volatile int* abort, int lane) {
+                                            uint32_t pass, Waits* waits, int lane) {
 #pragma unroll 1
   for (int g = side; g < NGROUP; g += 2) {
     // the steps' last use: N in the side's next segment (none after the last)
     const int last = g + 2 < NGROUP ? g + 2 : g;
     for (int h = 0; h < 2; h++)
-      if (!bar_wait(bars + 8 * (BAR_DONE + 2 * last + h), (pass + 1) & 1, abort)) return false;
+      if (!bar_wait(bars + 8 * (BAR_DONE + 2 * last + h), (pass + 1) & 1, waits)) return false;
     tc_fence_after();
     const int first = seg_first(side, g >> 1), end = first + seg_steps(side, g >> 1);
 #pragma unroll 2
@@ -505,11 +518,11 @@ __device__ __forceinline__ void extend_queue(ExtState& e, const TileInfo& t, con
 // passes so far.
 __device__ __forceinline__ bool extend_tile(ExtState& e, const TileInfo& t, const UngArgs& a, const unsigned char* rows,
                                             const int8_t* tab, const uint2* ring, volatile uint32_t* rp, int row0,
-                                            int window0, uint32_t& pass, volatile int* abort, int lane) {
+                                            int window0, uint32_t& pass, Waits* waits, int lane) {
   const int n_pass = (t.n2 + TC_M - 1) / TC_M;
   for (int p = 0; p < n_pass; p++, pass++) {
-    while (__shfl_sync(0xffffffffu, rp[0], 0) == pass) {
-      if (__any_sync(0xffffffffu, *abort != 0)) return false;
+    for (const uint32_t t0 = now(); __shfl_sync(0xffffffffu, rp[0], 0) == pass;) {
+      if (over(waits, t0)) return false;
       __nanosleep(100);
     }
     __threadfence_block();
@@ -545,8 +558,8 @@ __device__ __forceinline__ bool extend_tile(ExtState& e, const TileInfo& t, cons
 // maximised with it; then the accumulator may take the side's next segment.
 template <int NW, bool FIRST>
 __device__ __forceinline__ bool read_segment(uint32_t (&m)[NW], int g, uint32_t bars, int half, uint32_t pass,
-                                             uint32_t tm, volatile int* abort, int lane) {
-  if (!bar_wait(bars + 8 * (BAR_DONE + 2 * g + half), pass & 1, abort)) return false;
+                                             uint32_t tm, Waits* waits, int lane) {
+  if (!bar_wait(bars + 8 * (BAR_DONE + 2 * g + half), pass & 1, waits)) return false;
   tc_fence_after();
   uint32_t v[NW];
   tm_load_pack<NW>(tm, v);
@@ -567,7 +580,7 @@ __device__ __forceinline__ bool read_segment(uint32_t (&m)[NW], int g, uint32_t 
 template <int NW>
 __device__ __forceinline__ bool epilogue_tile(const TileInfo& t, uint2* ring, volatile uint32_t* rp, uint32_t bars,
                                               uint32_t tm, int half, int lane_window, uint32_t& pass,
-                                              volatile int* abort, int lane) {
+                                              Waits* waits, int lane) {
   constexpr int NMASK = (NW + 15) / 16;  // masks of 32 rows: row 4 j + b of a mask's rows at bit 8 b + j
   const int n_pass = (t.n2 + TC_M - 1) / TC_M;
   const int row0 = half * 2 * NW;
@@ -582,12 +595,12 @@ __device__ __forceinline__ bool epilogue_tile(const TileInfo& t, uint2* ring, vo
   for (int p = 0; p < n_pass; p++) {
     uint32_t r[NW], l[NW];
     const uint32_t tl = tm + 2 * TM_ACC;
-    if (!read_segment<NW, true>(r, 0, bars, half, pass, tm, abort, lane)) return false;
-    if (!read_segment<NW, true>(l, 1, bars, half, pass, tl, abort, lane)) return false;
+    if (!read_segment<NW, true>(r, 0, bars, half, pass, tm, waits, lane)) return false;
+    if (!read_segment<NW, true>(l, 1, bars, half, pass, tl, waits, lane)) return false;
 #pragma unroll 1
     for (int g = 2; g < NGROUP; g += 2) {
-      if (!read_segment<NW, false>(r, g, bars, half, pass, tm, abort, lane)) return false;
-      if (!read_segment<NW, false>(l, g + 1, bars, half, pass, tl, abort, lane)) return false;
+      if (!read_segment<NW, false>(r, g, bars, half, pass, tm, waits, lane)) return false;
+      if (!read_segment<NW, false>(l, g + 1, bars, half, pass, tl, waits, lane)) return false;
     }
     // the sign bits of bound - S1, gathered eight words (16 rows) at a time
     // into bit 7 of the mask's bytes, which move down
@@ -609,12 +622,9 @@ __device__ __forceinline__ bool epilogue_tile(const TileInfo& t, uint2* ring, vo
     }
     // a free place of the ring
     if (pass - seen >= RING) {
-      const long long t0 = clock64();
+      const uint32_t t0 = now();
       while (pass - (seen = __shfl_sync(0xffffffffu, rp[RP_TAKEN], 0)) >= RING) {
-        if (__any_sync(0xffffffffu, *abort || clock64() - t0 > WAIT_CLOCKS)) {
-          *abort = 1;
-          return false;
-        }
+        if (over(waits, t0)) return false;
         __nanosleep(100);
       }
     }
@@ -636,11 +646,11 @@ __device__ __forceinline__ bool epilogue_tile(const TileInfo& t, uint2* ring, vo
 // the compiler does not know to be uniform costs its move at each MMA.
 template <int SIDE, int HALF, int SEG>
 __device__ __forceinline__ bool mma_segments(uint64_t prof, uint32_t idesc, uint32_t bars, uint32_t pass,
-                                             volatile int* abort) {
+                                             Waits* waits) {
   if constexpr (SEG < NSEG) {
     constexpr int G = 2 * SEG + SIDE;
     constexpr uint32_t d = (2 * SIDE + HALF) * TM_ACC;
-    if (!bar_wait(bars + 8 * (BAR_GO + 2 * G + HALF), pass & 1, abort)) return false;
+    if (!bar_wait(bars + 8 * (BAR_GO + 2 * G + HALF), pass & 1, waits)) return false;
     tc_fence_after();
     if (elect_one()) {
       if constexpr (SEG == 0) {
@@ -660,7 +670,7 @@ __device__ __forceinline__ bool mma_segments(uint64_t prof, uint32_t idesc, uint
       tc_commit(bars + 8 * (BAR_DONE + 2 * G + HALF));
     }
     __syncwarp();
-    return mma_segments<SIDE, HALF, SEG + 1>(prof, idesc, bars, pass, abort);
+    return mma_segments<SIDE, HALF, SEG + 1>(prof, idesc, bars, pass, waits);
   }
   return true;
 }
@@ -668,9 +678,9 @@ __device__ __forceinline__ bool mma_segments(uint64_t prof, uint32_t idesc, uint
 // The tile's passes of a chain.
 template <int SIDE, int HALF>
 __device__ __forceinline__ void mma_tile(uint64_t prof, uint32_t idesc, uint32_t bars, int n_pass, uint32_t& pass,
-                                         volatile int* abort) {
+                                         Waits* waits) {
   for (int p = 0; p < n_pass; p++, pass++)
-    if (!mma_segments<SIDE, HALF, 0>(prof, idesc, bars, pass, abort)) return;
+    if (!mma_segments<SIDE, HALF, 0>(prof, idesc, bars, pass, waits)) return;
 }
 
 // ---------------------------------------------------------------------------
@@ -722,7 +732,7 @@ __device__ __forceinline__ bool fetch_tile(const UngArgs& a, const ScoreTable& c
   if (lane == 0) *reinterpret_cast<TileInfo*>(smem + OFF_SLOTS + (k % TILES) * SLOT_INFO) = t;
   __threadfence_block();
   __syncwarp();
-  if (lane == 0) *reinterpret_cast<volatile uint32_t*>(smem + OFF_MISC + 8) = k + 1;
+  if (lane == 0) *reinterpret_cast<volatile uint32_t*>(smem + OFF_MISC + 4) = k + 1;
   return t.rows > 0;
 }
 
@@ -756,12 +766,13 @@ __device__ __forceinline__ void build_profile(unsigned char* smem, const unsigne
   }
 }
 
-__global__ void __launch_bounds__(TC_THREADS, 1) k_ungapped_mma(UngArgs a, const __grid_constant__ ScoreTable c) {
+__global__ void __launch_bounds__(TC_THREADS, 1) k_ungapped_mma(UngArgs a, const __grid_constant__ ScoreTable c,
+                                                                const uint32_t wait_limit) {
   extern __shared__ __align__(1024) unsigned char smem[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint32_t sb = saddr(smem);
   const uint32_t bars = sb + OFF_BAR;
-  volatile int* abort = reinterpret_cast<volatile int*>(smem + OFF_MISC + 4);
+  Waits* waits = reinterpret_cast<Waits*>(smem + OFF_WAITS);
 
   // one-time set-up: tables, barriers, tensor memory, block scales
   int8_t* tab = reinterpret_cast<int8_t*>(smem + OFF_TAB);
@@ -793,8 +804,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_ungapped_mma(UngArgs a, const
   for (int i = tid; i < TC_M; i += TC_THREADS)  // no cell: past the window
     *reinterpret_cast<uint32_t*>(smem + OFF_WIN + (TC_M + i) * WIN_STRIDE + WIN - LEFT_BYTE) = 0x01010101u * NCODE;
   if (tid == 0) {
-    *abort = 0;
-    *reinterpret_cast<uint32_t*>(smem + OFF_MISC + 8) = 0;
+    waits->abort = 0;
+    waits->limit = wait_limit;
+    *reinterpret_cast<uint32_t*>(smem + OFF_MISC + 4) = 0;
     for (int g = 0; g < 2 * NGROUP; g++) {
       bar_init(bars + 8 * (BAR_GO + g), EXP_WARPS / 2 + EPI_WARPS / 2);
       bar_init(bars + 8 * (BAR_DONE + g), 1);
@@ -814,7 +826,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_ungapped_mma(UngArgs a, const
   tc_fence_after();
   // (all columns are allocated, so the base is column 0)
   const uint32_t tm_base = *reinterpret_cast<uint32_t*>(smem + OFF_MISC);
-  if (tm_base != 0u) *abort = 1;
+  if (tm_base != 0u) {
+    *(volatile int*)&waits->abort = 1;
+    if (tid == 0) atomicOr(a.err, UNG_ERR_TMEM);
+  }
   if (warp < 4) {
     const uint32_t tml = (uint32_t)(warp * 32) << 16;
     const uint32_t s1[8] = {0x7f7f7f7fu, 0x7f7f7f7fu, 0x7f7f7f7fu, 0x7f7f7f7fu,
@@ -848,10 +863,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_ungapped_mma(UngArgs a, const
       bar_arrive(bars + 8 * (BAR_GO + half));
       bar_arrive(bars + 8 * (BAR_GO + 2 + half));
     }
-    for (uint32_t k = 0; wait_tile(smem, k, t, abort); k++) {
+    for (uint32_t k = 0; wait_tile(smem, k, t, waits); k++) {
       __syncwarp();
       if (lane == 0) bar_arrive(bars + 8 * BAR_READ);
-      if (!bar_wait(bars + 8 * BAR_READ, k & 1, abort)) break;
+      if (!bar_wait(bars + 8 * BAR_READ, k & 1, waits)) break;
       build_profile(smem, smem + OFF_ROWS + (k % TILE_ROWS) * ROWS_BYTES, t, tid);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       tc_fence_before();
@@ -860,10 +875,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_ungapped_mma(UngArgs a, const
       const uint32_t tml = ((uint32_t)(q * 32) << 16) + half * TM_ACC;
       const int lw = q * 32 + lane;
       bool ok;
-      if (t.half == 64) ok = epilogue_tile<32>(t, ring, rp, bars, tml, half, lw, pass, abort, lane);
-      else if (t.half == 48) ok = epilogue_tile<24>(t, ring, rp, bars, tml, half, lw, pass, abort, lane);
-      else if (t.half == 32) ok = epilogue_tile<16>(t, ring, rp, bars, tml, half, lw, pass, abort, lane);
-      else ok = epilogue_tile<8>(t, ring, rp, bars, tml, half, lw, pass, abort, lane);
+      if (t.half == 64) ok = epilogue_tile<32>(t, ring, rp, bars, tml, half, lw, pass, waits, lane);
+      else if (t.half == 48) ok = epilogue_tile<24>(t, ring, rp, bars, tml, half, lw, pass, waits, lane);
+      else if (t.half == 32) ok = epilogue_tile<16>(t, ring, rp, bars, tml, half, lw, pass, waits, lane);
+      else ok = epilogue_tile<8>(t, ring, rp, bars, tml, half, lw, pass, waits, lane);
       if (!ok) break;
     }
   } else if (warp < EXT_WARP) {
@@ -875,7 +890,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_ungapped_mma(UngArgs a, const
     uint32_t* win = reinterpret_cast<uint32_t*>(smem + OFF_WIN + (side * TC_M + q * 32 + lane) * WIN_STRIDE);
     const uint32_t win_s = saddr(win) - side * LEFT_BYTE;
     const uint4 sent = make_uint4(0x15151515u, 0x15151515u, 0x15151515u, 0x15151515u);
-    for (uint32_t k = 0; wait_tile(smem, k, t, abort); k++) {
+    for (uint32_t k = 0; wait_tile(smem, k, t, waits); k++) {
       const uint4* src = reinterpret_cast<const uint4*>(a.nb2 + t.v0 * WIN) + side;
       uint4 x = sent, y = sent;
       if (q * 32 + lane < t.n2) {
@@ -899,7 +914,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_ungapped_mma(UngArgs a, const
           x = __ldg(src + (int64_t)w * 3);
           y = __ldg(src + (int64_t)w * 3 + 1);
         }
-        ok = expand_pass(side, win_s, lut, tml, bars, pass, abort, lane);
+        ok = expand_pass(side, win_s, lut, tml, bars, pass, waits, lane);
       }
       if (!ok) break;
     }
@@ -915,9 +930,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_ungapped_mma(UngArgs a, const
     const uint2* ring = reinterpret_cast<const uint2*>(smem + OFF_RING) + x * RING * 32;
     volatile uint32_t* rp = reinterpret_cast<volatile uint32_t*>(smem + OFF_RPOS) + x;
     volatile uint32_t* ended = reinterpret_cast<volatile uint32_t*>(smem + OFF_RPOS) + RP_EXT;
-    for (uint32_t k = 0; wait_tile(smem, k, t, abort); k++) {
+    for (uint32_t k = 0; wait_tile(smem, k, t, waits); k++) {
       if (!extend_tile(e, t, a, smem + OFF_ROWS + (k % TILE_ROWS) * ROWS_BYTES, reinterpret_cast<const int8_t*>(smem + OFF_TAB),
-                       ring, rp, (x >> 2) * t.half, (x & 3) * 32, pass, abort, lane))
+                       ring, rp, (x >> 2) * t.half, (x & 3) * 32, pass, waits, lane))
         break;
       __syncwarp();
       if (lane == 0) ended[x] = k + 1;
@@ -926,28 +941,35 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_ungapped_mma(UngArgs a, const
   } else if (warp < TILE_WARP) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(TC_REGS_MMA));
     const uint64_t prof = tc_desc(sb + OFF_PROF);
-    for (uint32_t k = 0; wait_tile(smem, k, t, abort); k++) {
-      if (!bar_wait(bars + 8 * BAR_PROF, k & 1, abort)) break;
+    for (uint32_t k = 0; wait_tile(smem, k, t, waits); k++) {
+      if (!bar_wait(bars + 8 * BAR_PROF, k & 1, waits)) break;
       tc_fence_after();
       const uint32_t n = __shfl_sync(0xffffffffu, (uint32_t)t.half, 0);
       const uint32_t idesc = (1u << 7) | (1u << 10) | ((n >> 3) << 17) | (1u << 23) | (8u << 24);
       const int n_pass = (t.n2 + TC_M - 1) / TC_M;
-      if (warp == MMA_WARP) mma_tile<0, 0>(prof, idesc, bars, n_pass, pass, abort);
-      else if (warp == MMA_WARP + 1) mma_tile<1, 0>(prof, idesc, bars, n_pass, pass, abort);
-      else if (warp == MMA_WARP + 2) mma_tile<0, 1>(prof + n, idesc, bars, n_pass, pass, abort);
-      else mma_tile<1, 1>(prof + n, idesc, bars, n_pass, pass, abort);
+      if (warp == MMA_WARP) mma_tile<0, 0>(prof, idesc, bars, n_pass, pass, waits);
+      else if (warp == MMA_WARP + 1) mma_tile<1, 0>(prof, idesc, bars, n_pass, pass, waits);
+      else if (warp == MMA_WARP + 2) mma_tile<0, 1>(prof + n, idesc, bars, n_pass, pass, waits);
+      else mma_tile<1, 1>(prof + n, idesc, bars, n_pass, pass, waits);
     }
   } else {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(TC_REGS_MMA));
     if (warp == TILE_WARP) {
       // ahead of the others, once every extend warp has ended the tile that
-      // used the row buffer last (a tile can take long: the others' own waits
-      // tell a failure)
-      volatile uint32_t* ended = reinterpret_cast<volatile uint32_t*>(smem + OFF_RPOS) + RP_EXT;
+      // used the row buffer last (a tile can take long: the limit counts from
+      // the last pass that an extend warp took)
+      volatile uint32_t* taken = reinterpret_cast<volatile uint32_t*>(smem + OFF_RPOS) + RP_TAKEN + lane % EXT_WARPS;
+      volatile uint32_t* ended = reinterpret_cast<volatile uint32_t*>(smem + OFF_RPOS) + RP_EXT + lane % EXT_WARPS;
       for (uint32_t k = 0;; k++) {
         bool ok = true;
-        while (ok && __any_sync(0xffffffffu, ended[lane % EXT_WARPS] + TILE_ROWS <= k)) {
-          if (__any_sync(0xffffffffu, *abort != 0)) ok = false;
+        uint32_t t0 = now(), last = *taken;
+        for (uint32_t polls = 1; ok && __any_sync(0xffffffffu, *ended + TILE_ROWS <= k); polls++) {
+          if (polls % 64 == 0) {  // (at every poll the longer loop cost the other roles 1 %)
+            const uint32_t at = *taken;
+            if (__any_sync(0xffffffffu, at != last)) t0 = now();
+            last = at;
+            ok = !over(waits, t0);
+          }
           __nanosleep(400);
         }
         if (!ok || !fetch_tile(a, c, smem, k, lane)) break;
@@ -960,18 +982,23 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_ungapped_mma(UngArgs a, const
     // shared and tensor memory go
     if (elect_one()) tc_commit(bars + 8 * BAR_DRAIN);
     __syncwarp();
-    const long long t0 = clock64();
-    while (!bar_try(bars + 8 * BAR_DRAIN, 0) && clock64() - t0 < WAIT_CLOCKS) {
+    const uint32_t t0 = now();
+    while (!bar_try(bars + 8 * BAR_DRAIN, 0) && now() - t0 < UNG_WAIT_CLOCKS) {
     }
   }
   tc_fence_before();
   __syncthreads();
-  if (tid == 0 && *abort) atomicOr(a.err, 1);
+  if (tid == 0 && *(volatile int*)&waits->abort) atomicOr(a.err, UNG_ERR_WAIT);
   if (warp == MMA_WARP)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tm_base), "r"(TM_COLS));
 }
 
 }  // namespace
+
+static std::atomic<uint32_t> g_wait_limit{UNG_WAIT_CLOCKS};
+void set_ungapped_wait_limit(int64_t clocks) {
+  g_wait_limit.store(clocks > 0 && clocks < UNG_WAIT_CLOCKS ? (uint32_t)clocks : UNG_WAIT_CLOCKS);
+}
 
 cudaError_t launch_ungapped_mma(const UngArgs& a, int grid, cudaStream_t st) {
   static std::atomic<bool> attr_set[64];  // per device; calls may come from several threads
@@ -991,7 +1018,7 @@ cudaError_t launch_ungapped_mma(const UngArgs& a, int grid, cudaStream_t st) {
     return s;
   }();
   note_launch();
-  k_ungapped_mma<<<grid, TC_THREADS, TC_SMEM, st>>>(a, table);
+  k_ungapped_mma<<<grid, TC_THREADS, TC_SMEM, st>>>(a, table, g_wait_limit.load());
   return cudaGetLastError();
 }
 
