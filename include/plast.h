@@ -423,15 +423,20 @@ int plast_get_tile_costs(plast_tile_costs* out);
 int plast_set_tile_costs(const plast_tile_costs* costs);
 int plast_set_tile_shape(int mode);
 /*
- * The stage-2 work list, every wide tile charged as a full one, of two banks with
- * the given CSR key offsets (host arrays of PLAST_NKEYS + 1 entries each, as
- * plast_bank_export_index returns) on a GPU of n_sms SMs (0: no splitting of
- * long lists): host-only, no device needed.  Fills tiles[6 * t ..] with (key,
+ * plast_stage2_tiles_at: the work list that stage 2 at threshold s1 runs, under
+ * the current schedule, costs and tile shape, for two banks with the given CSR
+ * key offsets (host arrays of PLAST_NKEYS + 1 entries each, as
+ * plast_bank_export_index returns) on a GPU of n_sms SMs (0: long lists stay
+ * whole, and each key's remainder goes by cost alone): host-only, no device
+ * needed.  plast_stage2_tiles: the list by the plain form of the cost model,
+ * which depends on no threshold: every wide tile is charged as a full one.  Fills tiles[6 * t ..] with (key,
  * first bank-1 CSR index, rows, shape: 0 wide, 1, 2, 3, 4 narrow of 8, 4, 2,
  * 16 rows, first and end offset of its bank-2 windows in the key's list) in
  * launch order for t < *n_tiles; PLAST_E_CAPACITY if more than `cap` tiles
  * (then *n_tiles = needed), PLAST_E_INVALID on decreasing offsets.
  */
+int plast_stage2_tiles_at(const int64_t* key_off1, const int64_t* key_off2, int32_t s1, int32_t n_sms, int32_t* tiles,
+                          int64_t cap, int64_t* n_tiles);
 int plast_stage2_tiles(const int64_t* key_off1, const int64_t* key_off2, int32_t n_sms, int32_t* tiles, int64_t cap,
                        int64_t* n_tiles);
 

@@ -142,6 +142,8 @@ def lib() -> ctypes.CDLL:
         L.plast_set_tile_costs.restype = ctypes.c_int
         L.plast_stage2_tiles.argtypes = [P, P, i32, P, i64, pI64]
         L.plast_stage2_tiles.restype = ctypes.c_int
+        L.plast_stage2_tiles_at.argtypes = [P, P, i32, i32, P, i64, pI64]
+        L.plast_stage2_tiles_at.restype = ctypes.c_int
         L.plast_set_tile_shape.argtypes = [ctypes.c_int]
         L.plast_set_tile_shape.restype = ctypes.c_int
         L.plast_set_timing.argtypes = [ctypes.c_int]
@@ -262,10 +264,13 @@ def plast_set_tile_shape(mode: int) -> None:
         raise PlastError("plast_set_tile_shape", rc)
 
 
-def plast_stage2_tiles(key_off1: np.ndarray, key_off2: np.ndarray, n_sms: int = 0) -> np.ndarray:
+def plast_stage2_tiles(key_off1: np.ndarray, key_off2: np.ndarray, n_sms: int = 0,
+                       s1: int | None = None) -> np.ndarray:
     """Host-only: the stage-2 tiles [t, 6] = (key, first bank-1 CSR index,
     rows, shape, first and end bank-2 offset in the key's list) for two
-    banks' CSR key offsets, long lists cut for a GPU of ``n_sms`` SMs."""
+    banks' CSR key offsets, long lists cut for a GPU of ``n_sms`` SMs: with
+    ``s1`` the list that stage 2 at that threshold runs, without it the list
+    with every wide tile charged as a full one."""
     k1 = np.ascontiguousarray(key_off1, dtype=np.int64)
     k2 = np.ascontiguousarray(key_off2, dtype=np.int64)
     if len(k1) != NKEYS + 1 or len(k2) != NKEYS + 1:
@@ -274,8 +279,9 @@ def plast_stage2_tiles(key_off1: np.ndarray, key_off2: np.ndarray, n_sms: int = 
     cap = 0
     for _ in range(2):
         out = np.zeros((max(cap, 1), 6), dtype=np.int32)
-        rc = lib().plast_stage2_tiles(k1.ctypes.data, k2.ctypes.data, int(n_sms), out.ctypes.data, cap,
-                                      ctypes.byref(n))
+        at = (out.ctypes.data, cap, ctypes.byref(n))
+        rc = (lib().plast_stage2_tiles(k1.ctypes.data, k2.ctypes.data, int(n_sms), *at) if s1 is None else
+              lib().plast_stage2_tiles_at(k1.ctypes.data, k2.ctypes.data, int(s1), int(n_sms), *at))
         if rc == PLAST_E_CAPACITY:
             cap = n.value
             continue

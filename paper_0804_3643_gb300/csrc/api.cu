@@ -510,7 +510,7 @@ void build_tiles(const plast_bank* b1, const plast_bank* b2, bool largest_first,
 
 // The tensor kernel extends the pairs its bound lets through, so it pays at
 // thresholds that few pairs reach.
-bool stage2_on_tensor(const plast_params& prm) { return prm.s1 >= UNG_TC_MIN_S1; }
+bool stage2_on_tensor(int32_t s1) { return s1 >= UNG_TC_MIN_S1; }
 
 // The survivor rate of the last stage 2 of each pair of banks at each threshold
 // over each choice of keys, to size the next one's survivor buffer.  The first guess, pairs /
@@ -583,7 +583,7 @@ int run_ungapped(const plast_bank* b1, const plast_bank* b2, const plast_params&
   sv->sh = b2->pad_bits;
   TileList tl;
   const int mode = g_schedule.load();
-  build_tiles(b1, b2, mode == 0, &tl, stage2_on_tensor(prm), key_mask);
+  build_tiles(b1, b2, mode == 0, &tl, stage2_on_tensor(prm.s1), key_mask);
   t_timer.mark(0, st);
   if (tl.tiles.empty()) return PLAST_OK;
   const int64_t nt = (int64_t)tl.tiles.size();
@@ -1383,7 +1383,7 @@ int plast_plan_create(const plast_bank* b1, const plast_bank* b2, const plast_pa
     return rc_of(e);
   };
   TileList& tl = p->tl;
-  build_tiles(b1, b2, true, &tl, stage2_on_tensor(p->prm));
+  build_tiles(b1, b2, true, &tl, stage2_on_tensor(p->prm.s1));
   p->n_tiles = (int64_t)tl.tiles.size();
   cudaError_t e;
   auto alloc = [&](void** q, size_t bytes) { return dev_alloc(q, bytes < 16 ? 16 : bytes); };
@@ -1690,8 +1690,9 @@ int plast_set_tile_costs(const plast_tile_costs* c) {
   return PLAST_OK;
 }
 
-int plast_stage2_tiles(const int64_t* key_off1, const int64_t* key_off2, int32_t n_sms, int32_t* tiles, int64_t cap,
-                       int64_t* n_tiles) {
+// tensor, listed: as build_tiles_from
+static int list_tiles(const int64_t* key_off1, const int64_t* key_off2, bool tensor, bool listed, int32_t n_sms,
+                      int32_t* tiles, int64_t cap, int64_t* n_tiles) {
   if (!key_off1 || !key_off2 || !n_tiles || cap < 0 || n_sms < 0 || (cap > 0 && !tiles)) return PLAST_E_INVALID;
   for (int k = 0; k < NKEYS; k++)
     if (key_off1[k + 1] < key_off1[k] || key_off2[k + 1] < key_off2[k] || key_off1[k + 1] > INT32_MAX ||
@@ -1699,7 +1700,7 @@ int plast_stage2_tiles(const int64_t* key_off1, const int64_t* key_off2, int32_t
       return PLAST_E_INVALID;
   TileList tl;
   const bool persistent = g_schedule.load() == 0;
-  build_tiles_from(key_off1, key_off2, persistent, &tl, nullptr, -1, persistent ? n_sms : 0, false, true);
+  build_tiles_from(key_off1, key_off2, persistent, &tl, nullptr, -1, persistent ? n_sms : 0, tensor, listed);
   *n_tiles = (int64_t)tl.tiles.size();
   if (*n_tiles > cap) return PLAST_E_CAPACITY;
   for (size_t i = 0; i < tl.tiles.size(); i++) {
@@ -1713,6 +1714,16 @@ int plast_stage2_tiles(const int64_t* key_off1, const int64_t* key_off2, int32_t
     o[5] = t.w;
   }
   return PLAST_OK;
+}
+
+int plast_stage2_tiles(const int64_t* key_off1, const int64_t* key_off2, int32_t n_sms, int32_t* tiles, int64_t cap,
+                       int64_t* n_tiles) {
+  return list_tiles(key_off1, key_off2, false, true, n_sms, tiles, cap, n_tiles);
+}
+
+int plast_stage2_tiles_at(const int64_t* key_off1, const int64_t* key_off2, int32_t s1, int32_t n_sms, int32_t* tiles,
+                          int64_t cap, int64_t* n_tiles) {
+  return list_tiles(key_off1, key_off2, stage2_on_tensor(s1), false, n_sms, tiles, cap, n_tiles);
 }
 
 int plast_set_tile_shape(int mode) {
