@@ -11,6 +11,7 @@
 #include <atomic>
 #include <mutex>
 #include <new>
+#include <numeric>
 #include <stdio.h>
 #include <string.h>
 #include <vector>
@@ -144,9 +145,9 @@ int num_sms() {
 
 // Stage-2 tile costs in SM-nanoseconds: per slot (a bank-1 row of the tile's
 // shape against a bank-2 window: 48 cells, whatever the tile's fill) and per
-// tile.  A CTA moves through a key's bank-2 windows a pass at a time (32 warps
-// x 4 windows wide, x 32 narrow), so a tile is charged its shape's rows x n2
-// rounded up to that granularity.  Defaults from a GB300; plast_autotune
+// tile.  A CTA moves through a key's bank-2 windows a pass at a time (wide: 128
+// windows on the tensor cores, 96 in the plain kernel; narrow: 512), so a tile
+// is charged its shape's rows x n2 rounded up to that granularity.  Defaults from a GB300; plast_autotune
 // measures them on the current device.  The wide costs are the tensor
 // kernel's, whose pass costs (rows rounded up to 32) + TC_FIXED_ROWS (measured:
 // 1.23, 1.5, 2.0 and 2.29 SM-microseconds a pass of 32, 64, 96 and 128 rows);
@@ -164,8 +165,6 @@ std::mutex g_cost_mu;
 plast_tile_costs g_costs = {0.140, 3660.0, 0.352, 729.0, 0.409, 783.0, 0.565, 831.0, 12, 0, 0.323, 383.0};
 // 0: by cost; 1: wide only; 2, 3, 4, 5: narrow tiles of 8, 4, 2, 16 rows only
 std::atomic<int> g_shape{0};
-constexpr int64_t WIDE_PASS = 128;                         // bank-2 windows per CTA pass, wide tile
-constexpr int64_t NARROW_PASS = UNG_NARROW_PASS;           // narrow tiles
 int64_t round_up(int64_t n, int64_t g) { return (n + g - 1) / g * g; }
 
 int shape_rows(int shape) {
@@ -183,28 +182,52 @@ int shape_rows(int shape) {
   }
 }
 
-// Slots a tile is charged for; rows: of a wide tile of the tensor kernel, the
-// rows it holds (a full tile's share of what its passes cost).
-double shape_slots(int shape, int64_t n2, int64_t rows = UNG_T1) {
-  const double full = (double)shape_rows(shape) * (double)round_up(n2, shape == UNG_WIDE ? WIDE_PASS : NARROW_PASS);
-  if (shape != UNG_WIDE || rows == UNG_T1) return full;
-  return full * (double)(round_up(rows, 32) + TC_FIXED_ROWS) / (double)(UNG_T1 + TC_FIXED_ROWS);
-}
-
-double tile_cost(const plast_tile_costs& c, int shape, int64_t n2, int64_t rows = UNG_T1) {
-  const double slots = shape_slots(shape, n2, rows);
-  switch (shape) {
-    case UNG_WIDE:
-      return c.wide_slot * slots + c.wide_tile;
-    case UNG_NARROW:
-      return c.narrow_slot * slots + c.narrow_tile;
-    case UNG_NARROW4:
-      return c.narrow4_slot * slots + c.narrow4_tile;
-    case UNG_NARROW16:
-      return c.narrow16_slot * slots + c.narrow16_tile;
-    default:
-      return c.narrow2_slot * slots + c.narrow2_tile;
+// What a tile costs, for one of the wide kernels.
+struct CostModel {
+  plast_tile_costs c;
+  int64_t wide_pass;  // bank-2 windows a CTA of the wide kernel scores per pass
+  bool partial;       // the tensor kernel's: a wide tile that is not full costs less
+  int64_t pass(int shape) const { return shape == UNG_WIDE ? wide_pass : (int64_t)UNG_NARROW_PASS; }
+  // Slots a tile of `rows` rows is charged for (a partial wide tile of the
+  // tensor kernel: a full one's share of what its passes cost).
+  double slots(int shape, int64_t n2, int64_t rows) const {
+    const double full = (double)shape_rows(shape) * (double)round_up(n2, pass(shape));
+    if (shape != UNG_WIDE || !partial) return full;
+    return full * (double)(round_up(rows, 32) + TC_FIXED_ROWS) / (double)(UNG_T1 + TC_FIXED_ROWS);
   }
+  double cost(int shape, int64_t n2, int64_t rows = UNG_T1) const {
+    const double n = slots(shape, n2, rows);
+    switch (shape) {
+      case UNG_WIDE:
+        return c.wide_slot * n + c.wide_tile;
+      case UNG_NARROW:
+        return c.narrow_slot * n + c.narrow_tile;
+      case UNG_NARROW4:
+        return c.narrow4_slot * n + c.narrow4_tile;
+      case UNG_NARROW16:
+        return c.narrow16_slot * n + c.narrow16_tile;
+      default:
+        return c.narrow2_slot * n + c.narrow2_tile;
+    }
+  }
+  double cost(const int4& t) const { return cost(tile_shape(t), (int64_t)t.w - t.z, tile_rows(t)); }
+};
+
+// tensor: the wide tiles are the tensor kernel's; listed: as plast_stage2_tiles
+// lists them, every wide tile charged as a full one.
+CostModel cost_model(bool tensor, bool listed = false) {
+  CostModel m;
+  {
+    std::lock_guard<std::mutex> lk(g_cost_mu);
+    m.c = g_costs;
+  }
+  m.partial = tensor;
+  m.wide_pass = tensor || listed ? UNG_TC_PASS : UNG_WIDE_PASS;
+  if (!tensor && !listed) {
+    m.c.wide_slot = PLAIN_WIDE_SLOT;
+    m.c.wide_tile = PLAIN_WIDE_TILE;
+  }
+  return m;
 }
 
 // Stage-2 work list: for every key present in both banks, tiles of
@@ -219,12 +242,6 @@ struct TileList {
   int64_t pairs = 0;
   bool tensor = false;            // the wide tiles are the tensor kernel's
 };
-
-// The rows a tile is charged for: a partial wide tile of the tensor kernel
-// costs less than a full one.
-int64_t charged_rows(const int4& t, bool tensor) {
-  return tensor && tile_shape(t) == UNG_WIDE ? tile_rows(t) : UNG_T1;
-}
 
 struct PlannedTile {
   double cost;
@@ -261,7 +278,7 @@ PlanLists& plan_lists() {
 // passes, so that no piece costs more than about 1/4 of a CTA's share, and the
 // pieces take their places costliest first.  v is one launch's tile list,
 // costliest first but for the partial wide tiles.
-void split_long_tiles(const plast_tile_costs& c, std::vector<PlannedTile>& v, int64_t ctas, bool tensor) {
+void split_long_tiles(const CostModel& m, std::vector<PlannedTile>& v, int64_t ctas) {
   if (v.empty() || ctas <= 0) return;
   double total = 0, largest = 0;
   for (const PlannedTile& t : v) total += t.cost, largest = std::max(largest, t.cost);
@@ -273,7 +290,7 @@ void split_long_tiles(const plast_tile_costs& c, std::vector<PlannedTile>& v, in
   for (const PlannedTile& x : v) {
     const int4 t = x.tile;
     const int shape = tile_shape(t);
-    const int64_t pass = shape == UNG_WIDE ? WIDE_PASS : NARROW_PASS, n2 = (int64_t)t.w - t.z;
+    const int64_t pass = m.pass(shape), n2 = (int64_t)t.w - t.z;
     const int64_t cuts =
         x.cost <= 2 * target ? 1 : std::min<int64_t>((int64_t)std::ceil(x.cost / target), (n2 + pass - 1) / pass);
     if (cuts < 2) {
@@ -284,7 +301,7 @@ void split_long_tiles(const plast_tile_costs& c, std::vector<PlannedTile>& v, in
     for (int64_t a = 0; a < n2; a += chunk) {
       const int4 p = make_tile(tile_key(t), t.y, tile_rows(t), shape, t.z + (int)a,
                                t.z + (int)std::min<int64_t>(a + chunk, n2));
-      pieces.push_back({tile_cost(c, shape, (int64_t)p.w - p.z, charged_rows(p, tensor)), p});
+      pieces.push_back({m.cost(p), p});
     }
   }
   if (!std::is_sorted(rest.begin(), rest.end(), costlier)) std::stable_sort(rest.begin(), rest.end(), costlier);
@@ -300,15 +317,7 @@ void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first
   tl->tensor = tensor;
   tl->pairs = 0;
   tl->n_wide = 0;
-  plast_tile_costs c;
-  {
-    std::lock_guard<std::mutex> lk(g_cost_mu);
-    c = g_costs;
-  }
-  if (!tensor && !listed) {
-    c.wide_slot = PLAIN_WIDE_SLOT;
-    c.wide_tile = PLAIN_WIDE_TILE;
-  }
+  const CostModel m = cost_model(tensor, listed);
   const int mode = shape_override >= 0 ? shape_override : g_shape.load();
   // Keys in launch order: the persistent schedule takes them by decreasing
   // n2, which orders the tiles of each shape by decreasing cost (a tile's
@@ -323,15 +332,16 @@ void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first
     keys.push_back(k);
   }
   if (largest_first) {
-    // counting sort by decreasing ceil(n2 / 128), the quantity every tile
-    // cost depends on (monotonically), stable in key order
+    // counting sort by decreasing n2 in steps that both kernels' passes are
+    // multiples of: every tile cost rises with it; stable in key order
+    const int64_t step = std::gcd(m.wide_pass, (int64_t)UNG_NARROW_PASS);
     int64_t bmax = 0;
     for (const int k : keys) bmax = std::max<int64_t>(bmax, ko2[k + 1] - ko2[k]);
-    const int NB = (int)std::min<int64_t>(round_up(bmax, WIDE_PASS) / WIDE_PASS + 1, 1 << 20);
+    const int NB = (int)std::min<int64_t>(round_up(bmax, step) / step + 1, 1 << 20);
     static thread_local std::vector<int32_t> count;
     count.assign((size_t)NB + 1, 0);
     auto bucket = [&](int k) {
-      const int64_t b = round_up(ko2[k + 1] - ko2[k], WIDE_PASS) / WIDE_PASS;
+      const int64_t b = round_up(ko2[k + 1] - ko2[k], step) / step;
       return NB - 1 - (int)std::min<int64_t>(b, NB - 1);
     };
     for (const int k : keys) count[bucket(k) + 1]++;
@@ -359,11 +369,11 @@ void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first
   bool full_wide = false;
   // a wide tile's cost for the current key: a pass's, by 32 rows, times its
   // passes
-  auto wide_cost = [&](int64_t rows) { return tile_cost(c, UNG_WIDE, n2_now, rows); };
+  auto wide_cost = [&](int64_t rows) { return m.cost(UNG_WIDE, n2_now, rows); };
   auto emit = [&](int k, int64_t first, int64_t rows, int shape, std::vector<PlannedTile>* lists_of_shape) {
     const int4 t = make_tile(k, (int)first, (int)rows, shape, 0, n2_now);
     if (out) out->push_back(t);
-    else if (shape == UNG_WIDE) wide.push_back({wide_cost(tensor ? rows : UNG_T1), t});
+    else if (shape == UNG_WIDE) wide.push_back({wide_cost(rows), t});
     else lists_of_shape[shape].push_back({cost_now[shape], t});
   };
   // Whether the rests that cost less as wide tiles become wide ones is known
@@ -374,9 +384,9 @@ void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first
     const int64_t n2 = ko2[k + 1] - ko2[k];
     tl->pairs += n1 * n2;
     n2_now = (int32_t)n2;
-    const bool new_passes = round_up(n2, NARROW_PASS) != cover_passes;
+    const bool new_passes = round_up(n2, UNG_NARROW_PASS) != cover_passes;
     if (new_passes)
-      for (int shape = UNG_NARROW; shape < UNG_SHAPES; shape++) cost_now[shape] = tile_cost(c, shape, n2);
+      for (int shape = UNG_NARROW; shape < UNG_SHAPES; shape++) cost_now[shape] = m.cost(shape, n2);
     int64_t u = ko1[k];
     const int64_t end = ko1[k + 1];
     if (mode >= 2) {  // one narrow shape only
@@ -390,7 +400,7 @@ void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first
     }
     const int64_t rem = end - u;
     if (new_passes && mode != 1) {
-      cover_passes = round_up(n2, NARROW_PASS);
+      cover_passes = round_up(n2, UNG_NARROW_PASS);
       best[0] = 0;
       pick[0] = 0;
       for (int t = 1; t < TAIL; t++) {
@@ -414,7 +424,7 @@ void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first
     const int64_t full = rem / br;
     const int tail = (int)(rem % br);
     const double narrow_cost = (double)full * cost_now[bulk] + best[tail];
-    const double gain = narrow_cost - wide_cost(tensor ? rem : UNG_T1);
+    const double gain = narrow_cost - wide_cost(rem);
     std::vector<PlannedTile>* to = by_shape;
     if (gain >= 0) {
       rests_gain += gain;
@@ -454,8 +464,8 @@ void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first
   merged(by_shape[UNG_NARROW2], by_shape[UNG_NARROW16], lists.half[1]);
   merged(lists.half[0], lists.half[1], narrow);
   if (n_sms > 0) {
-    split_long_tiles(c, wide, (int64_t)n_sms, tensor);
-    split_long_tiles(c, narrow, (int64_t)UNG_NARROW_CTAS_PER_SM * n_sms, tensor);
+    split_long_tiles(m, wide, (int64_t)n_sms);
+    split_long_tiles(m, narrow, (int64_t)UNG_NARROW_CTAS_PER_SM * n_sms);
   }
   tl->n_wide = (int64_t)wide.size();
   tl->tiles.reserve(wide.size() + narrow.size());
@@ -1590,9 +1600,8 @@ int time_stage2(const plast_bank* b1, const plast_bank* b2, int shape, bool tens
   CK(bank_wait(b2, st));
   build_tiles(b1, b2, true, &tl, tensor, nullptr, shape);
   *slots = 0;
-  for (const int4& t : tl.tiles) {
-    *slots += shape_slots(tile_shape(t), (int64_t)t.w - t.z, charged_rows(t, tensor));
-  }
+  const CostModel m = cost_model(tensor);
+  for (const int4& t : tl.tiles) *slots += m.slots(tile_shape(t), (int64_t)t.w - t.z, tile_rows(t));
   *tiles = (double)tl.tiles.size();
   *ms = 0;
   if (tl.tiles.empty()) return PLAST_OK;

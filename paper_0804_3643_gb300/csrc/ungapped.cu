@@ -105,6 +105,7 @@ constexpr int NT_WARPS = NT_THREADS / 32;
 constexpr int NWKEY_BYTES = NT_WARPS * WBUF * 8;           // 4096
 constexpr int NWVAL_BYTES = NT_WARPS * WBUF * 4;           // 2048
 static_assert(UNG_NARROW_PASS == NT_WARPS * 32, "narrow pass = one window per lane");
+static_assert(UNG_WIDE_PASS == NWARPS * 4, "wide pass = four windows per warp");
 static_assert(NPROF_BYTES % 16 == 0 && NROWS_BYTES % 16 == 0, "alignment");
 static_assert(Wide<UNG_MAX_N16>::SMEM <= 232448, "shared memory per CTA");
 

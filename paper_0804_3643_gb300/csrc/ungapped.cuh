@@ -63,6 +63,7 @@ void set_ungapped_wait_limit(int64_t clocks);
 constexpr int32_t UNG_ERR_WAIT = 1;  // a wait ran out
 constexpr int32_t UNG_ERR_TMEM = 2;  // tensor memory was not all the CTA's own
 constexpr int UNG_TC_PASS = 128;      // bank-2 windows the tensor kernel scores per pass
+constexpr int UNG_WIDE_PASS = UNG_THREADS / 32 * 4;  // and the plain wide kernel: four a warp
 // Lowest S1 whose wide tiles go to the tensor kernel: below it more pairs pass
 // the bound than their exact extension is worth (3,000 x 20,000 proteins, ms:
 // S1 = 38 1.81 against the plain kernel's 3.36, 34 2.54 / 3.50, 32 3.45 / 3.58,

@@ -126,3 +126,33 @@ def test_bad_offsets_at(costs):  # noqa: F811
     bad[10] = bad[11] + 1
     with pytest.raises(B.PlastError):
         B.plast_stage2_tiles(bad, k, s1=38)
+
+
+@pytest.mark.parametrize("s1,windows", [(31, 96), (-30000, 96), (32, 128)])
+def test_wide_pieces_are_whole_passes(costs, s1, windows):  # noqa: F811
+    # the plain wide kernel scores 96 windows a pass, the tensor kernel 128
+    rng = np.random.default_rng(19)
+    n1, n2 = np.zeros(NK, np.int64), rng.integers(1000, 200000, size=NK).astype(np.int64)
+    n1[rng.choice(NK, 200, replace=False)] = 128
+    B.plast_set_tile_shape(1)
+    tiles = B.plast_stage2_tiles(offsets(n1), offsets(n2), n_sms=152, s1=s1)
+    last = tiles[:, 5] == n2[tiles[:, 0]]
+    assert (tiles[:, 3] == WIDE).all() and (~last).sum() > 200
+    assert ((tiles[~last, 5] - tiles[~last, 4]) % windows == 0).all()
+    # costliest first: by passes
+    passes = -(-(tiles[:, 5] - tiles[:, 4]) // windows)
+    assert (np.diff(passes) <= 0).all()
+    # each row range's pieces partition its list
+    for k in np.unique(tiles[:, 0]):
+        v = sorted((int(a), int(b)) for a, b in tiles[tiles[:, 0] == k][:, 4:])
+        assert v[0][0] == 0 and v[-1][1] == n2[k] and all(a[1] == b[0] for a, b in zip(v, v[1:]))
+
+
+@pytest.mark.parametrize("s1", [31, 38])
+def test_narrow_order(costs, s1):  # noqa: F811
+    n1, n2 = random_counts(np.random.default_rng(20))
+    n2 += np.arange(NK) % 700 * (n2 > 0)  # list lengths at every step of both passes
+    tiles = B.plast_stage2_tiles(offsets(n1), offsets(n2), s1=s1)
+    narrow = tiles[tiles[:, 3] != WIDE]
+    cost = [tile_cost(costs, s, hi - lo) for _, _, _, s, lo, hi in narrow]
+    assert len(narrow) > 1000 and all(a >= b for a, b in zip(cost, cost[1:]))
