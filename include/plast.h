@@ -383,8 +383,8 @@ int plast_set_schedule(int mode);
 /*
  * Stage-2 tile shapes.  The work of a key is cut into tiles of consecutive
  * bank-1 occurrences: wide tiles of up to 128 rows (on the tensor cores for
- * thresholds s1 of 32 and more, by a packed int16 kernel below), and narrow tiles of 16, 8, 4 or 2 rows, one bank-2
- * window per lane, for short lists (a small query bank against a large one,
+ * thresholds s1 of 32 and more, by a packed int16 kernel below), and narrow
+ * tiles of 16, 8, 4 or 2 rows, one bank-2 window per lane, for short lists (a small query bank against a large one,
  * the end of a long list).  After the full wide tiles of a key, the library
  * covers the remainder either with one wide tile or with narrow tiles (16
  * rows while 16 or more remain, or 8 if those cost less per row, the last
@@ -392,15 +392,20 @@ int plast_set_schedule(int mode);
  * tile of shape S costs
  * S_slot x (rows of S) x ceil(n2 / P_S) x P_S + S_tile SM-nanoseconds, n2 the
  * key's bank-2 occurrences, P_S the bank-2 windows a CTA scores per pass
- * (128 wide, 512 narrow).  (On the tensor cores a wide tile that is not full
- * is charged (its rows rounded up to 32, plus 83) / 211 of the slots: a pass
- * has a fixed part worth 83 rows.)  plast_autotune measures the constants on the
+ * (512 narrow; wide 128 on the tensor cores, 96 in the int16 kernel).  On the
+ * tensor cores a wide tile that is not full is charged (its rows rounded up to
+ * 32, plus 83) / 211 of the slots, and without any full wide tile the remainders
+ * go there only if they save 30 SM-microseconds per SM together: both fixed.
+ * plast_autotune measures the constants on the
  * current device (random banks, the stage-2 kernel timed with every tile of
  * one shape, against a long and a short bank 2; about a second), installs
  * them and copies them to *out (may be NULL).  It also picks the variant of
- * the packed int16 wide kernel by timing each: how many cells of the wide profile are held as
- * int16 (no sign extension, twice the shared-memory traffic), then how many
- * passes ahead a warp fetches its next bank-2 windows (the staging depth).
+ * the packed int16 wide kernel by timing each: how many cells of the wide
+ * profile are held as int16 (no sign extension, twice the shared-memory
+ * traffic), then how many passes ahead a warp fetches its next bank-2 windows
+ * (the staging depth).  The wide costs are the tensor kernel's; the int16
+ * kernel's are measured and kept beside them, and costs that a caller sets
+ * scale both alike.
  * plast_get_tile_costs / plast_set_tile_costs read and install costs and
  * variant (for a cached calibration; PLAST_E_INVALID unless the slot costs
  * are positive, the tile costs non-negative, wide_int16_cells one of the

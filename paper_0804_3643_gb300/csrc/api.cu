@@ -151,8 +151,8 @@ int num_sms() {
 // measures them on the current device.  The wide costs are the tensor
 // kernel's, whose pass costs (rows rounded up to 32) + TC_FIXED_ROWS (measured:
 // 1.23, 1.5, 2.0 and 2.29 SM-microseconds a pass of 32, 64, 96 and 128 rows);
-// the plain wide kernel, which runs at an S1 below UNG_TC_MIN_S1, is charged
-// PLAIN_WIDE_SLOT for every row of the shape.
+// the plain wide kernel's, which runs at an S1 below UNG_TC_MIN_S1, stand in
+// the same proportion to them as when both were measured (g_plain).
 constexpr int TC_FIXED_ROWS = 83;
 // If no key fills a wide tile, the keys' rests go to the tensor kernel only when
 // together they save its launch and its ramps, WIDE_LAUNCH ns on every SM.
@@ -160,9 +160,13 @@ constexpr int TC_FIXED_ROWS = 83;
 // 0.200 ms, 187 x 20,000 0.346 / 0.318, 90 x 70,000 0.500 / 0.475, 187 x 70,000
 // 0.873 / 0.845; from 250 x 70,000 on the same.
 constexpr double WIDE_LAUNCH = 30000.0;
-constexpr double PLAIN_WIDE_SLOT = 0.317, PLAIN_WIDE_TILE = 2960.0;
 std::mutex g_cost_mu;
 plast_tile_costs g_costs = {0.140, 3660.0, 0.352, 729.0, 0.409, 783.0, 0.565, 831.0, 12, 0, 0.323, 383.0};
+// The plain wide kernel's costs, and the tensor kernel's measured beside them.
+struct PlainWide {
+  double slot, tile, tensor_slot, tensor_tile;
+};
+PlainWide g_plain = {0.317, 2960.0, 0.140, 3660.0};  // (under g_cost_mu)
 // 0: by cost; 1: wide only; 2, 3, 4, 5: narrow tiles of 8, 4, 2, 16 rows only
 std::atomic<int> g_shape{0};
 int64_t round_up(int64_t n, int64_t g) { return (n + g - 1) / g * g; }
@@ -217,15 +221,17 @@ struct CostModel {
 // lists them, every wide tile charged as a full one.
 CostModel cost_model(bool tensor, bool listed = false) {
   CostModel m;
+  PlainWide plain;
   {
     std::lock_guard<std::mutex> lk(g_cost_mu);
     m.c = g_costs;
+    plain = g_plain;
   }
   m.partial = tensor;
   m.wide_pass = tensor || listed ? UNG_TC_PASS : UNG_WIDE_PASS;
   if (!tensor && !listed) {
-    m.c.wide_slot = PLAIN_WIDE_SLOT;
-    m.c.wide_tile = PLAIN_WIDE_TILE;
+    m.c.wide_slot *= plain.slot / plain.tensor_slot;
+    m.c.wide_tile = plain.tensor_tile > 0 ? m.c.wide_tile * (plain.tile / plain.tensor_tile) : plain.tile;
   }
   return m;
 }
@@ -1777,6 +1783,7 @@ int plast_autotune(void* stream, plast_tile_costs* out) {
   const int saved_variant = ungapped_variant();
   double best_t = 0;
   int best_v = saved_variant;
+  PlainWide plain = {};
   // the plain wide kernel's variant: the int16 cells at staging depth 1, then
   // the staging depths of the best
   auto try_variant = [&](int v, bool first) {
@@ -1786,6 +1793,8 @@ int plast_autotune(void* stream, plast_tile_costs* out) {
     if (rc == PLAST_OK && (first || t_long < best_t)) {
       best_t = t_long;
       best_v = v;
+      plain.slot = slot;
+      plain.tile = tile;
       c.wide_int16_cells = ungapped_variant_n16(v);
       c.wide_stage_depth = ungapped_variant_depth(v);
     }
@@ -1810,7 +1819,14 @@ int plast_autotune(void* stream, plast_tile_costs* out) {
     return rc;
   }
   rc = plast_set_tile_costs(&c);
-  if (rc == PLAST_OK && out) *out = c;
+  if (rc != PLAST_OK) return rc;
+  plain.tensor_slot = c.wide_slot;
+  plain.tensor_tile = c.wide_tile;
+  {
+    std::lock_guard<std::mutex> lk(g_cost_mu);
+    g_plain = plain;
+  }
+  if (out) *out = c;
   return rc;
 }
 

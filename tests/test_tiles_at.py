@@ -156,3 +156,26 @@ def test_narrow_order(costs, s1):  # noqa: F811
     narrow = tiles[tiles[:, 3] != WIDE]
     cost = [tile_cost(costs, s, hi - lo) for _, _, _, s, lo, hi in narrow]
     assert len(narrow) > 1000 and all(a >= b for a, b in zip(cost, cost[1:]))
+
+
+@pytest.mark.parametrize("slot,tile", [(1.0, 1.0), (0.25, 1.0), (4.0, 1.0), (1.0, 12.0), (0.6, 3.0)])
+def test_callers_wide_costs_below_32(costs, slot, tile):  # noqa: F811
+    # the plain wide kernel's costs, 0.317 and 2,960 beside the tensor kernel's
+    # 0.140 and 3,660, scale with the wide costs that a caller sets
+    c = dict(costs, wide_slot=0.140 * slot, wide_tile=3660.0 * tile)
+    B.plast_set_tile_costs(c)
+    n1, n2 = random_counts(np.random.default_rng(21))
+    k1, k2 = offsets(n1), offsets(n2)
+    by_key = check_cover(B.plast_stage2_tiles(k1, k2, s1=31), k1, n1, n2)
+    wide_rests = narrow_rests = 0
+    for k, t in by_key.items():
+        t = sorted(t)
+        full, rem = divmod(int(n1[k]), T1)
+        if not rem:
+            continue
+        wide = 0.317 * slot * 128 * round_up(n2[k], 96) + 2960.0 * tile
+        goes_wide = narrow_cover(costs, rem, n2[k]) >= wide
+        assert ([s for _, _, s in t[full:]] == [WIDE]) == goes_wide
+        wide_rests += goes_wide
+        narrow_rests += not goes_wide
+    assert wide_rests > 50 and narrow_rests > 50
