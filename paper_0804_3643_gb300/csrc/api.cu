@@ -246,7 +246,7 @@ struct TileList {
   std::vector<int4> tiles;        // (key, first CSR index of bank 1, rows, shape)
   int64_t n_wide = 0;             // persistent order: the wide tiles come first
   int64_t pairs = 0;
-  bool tensor = false;            // the wide tiles are the tensor kernel's
+  bool tensor = false;            // the wide tiles are the tensor kernel's (key by key: of long lists)
 };
 
 struct PlannedTile {
@@ -323,7 +323,7 @@ void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first
   tl->tensor = tensor;
   tl->pairs = 0;
   tl->n_wide = 0;
-  const CostModel m = cost_model(tensor, listed);
+  const CostModel m = cost_model(tensor && largest_first, listed);
   const int mode = shape_override >= 0 ? shape_override : g_shape.load();
   // Keys in launch order: the persistent schedule takes them by decreasing
   // n2, which orders the tiles of each shape by decreasing cost (a tile's
@@ -430,7 +430,10 @@ void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first
     const int64_t full = rem / br;
     const int tail = (int)(rem % br);
     const double narrow_cost = (double)full * cost_now[bulk] + best[tail];
-    const double gain = narrow_cost - wide_cost(rem);
+    // (key by key a narrow launch after the key's wide one adds its whole
+    // length, a rest beside the full wide tiles nothing: see launch_tiles)
+    const bool beside = !largest_first && !listed && n1 >= UNG_T1;
+    const double gain = beside ? 0 : narrow_cost - wide_cost(rem);
     std::vector<PlannedTile>* to = by_shape;
     if (gain >= 0) {
       rests_gain += gain;
@@ -484,7 +487,14 @@ void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first
 // persistent schedule the wide kernel over the wide tiles and the narrow
 // kernel over the rest, each on its own counter (counters[0], counters[1],
 // zeroed by the caller); in the plain schedule, per key one launch of each
-// kernel its tiles need.
+// kernel its tiles need.  There each CTA of the tensor kernel pays its set-up
+// (tables, barriers, tensor memory: some 16 us more than the plain kernel's)
+// for one tile, so only keys with UNG_TC_KEY_WINDOWS bank-2 windows or more go
+// to it, and the plan is made with the plain kernel's costs.  Stage 2 key by
+// key, ms: with the plain kernel only and narrow rests / every wide tile on the
+// tensor kernel / this: batching stress (50,000 x 50,000) 927 / 980 / 857; a
+// tenth of it 189 / 265 / 164; 100,000 x 10,000 ordinary proteins 276 / 312 /
+// 224, 50,000 x 50,000 869 / 585 / 514, 10,000 x 100,000 1,561 / 878 / 796.
 cudaError_t launch_tiles(const TileList& tl, UngArgs a, int32_t* counters, bool persistent, cudaStream_t st) {
   const int64_t nt = (int64_t)tl.tiles.size();
   auto run = [&](int64_t lo, int64_t hi, bool wide, int32_t* counter) -> cudaError_t {
@@ -495,7 +505,8 @@ cudaError_t launch_tiles(const TileList& tl, UngArgs a, int32_t* counters, bool 
     a.persistent = persistent ? 1 : 0;
     const int per_sm = wide ? 1 : UNG_NARROW_CTAS_PER_SM;
     const int grid = persistent ? (int)std::min<int64_t>((int64_t)per_sm * num_sms(), hi - lo) : (int)(hi - lo);
-    if (wide && tl.tensor) return launch_ungapped_mma(a, grid, st);
+    if (wide && tl.tensor && (persistent || tl.tiles[lo].w >= UNG_TC_KEY_WINDOWS))
+      return launch_ungapped_mma(a, grid, st);
     return wide ? launch_ungapped(a, grid, st) : launch_ungapped_narrow(a, grid, st);
   };
   if (persistent) {

@@ -69,6 +69,11 @@ constexpr int UNG_WIDE_PASS = UNG_THREADS / 32 * 4;  // and the plain wide kerne
 // S1 = 38 1.81 against the plain kernel's 3.36, 34 2.54 / 3.50, 32 3.45 / 3.58,
 // 30 4.75 / 3.68).
 constexpr int UNG_TC_MIN_S1 = 32;
+// Fewest bank-2 windows of a key whose wide tiles go to the tensor kernel when
+// each key is a launch of its own (batching stress / 100,000 x 10,000 proteins,
+// ms: 512 904 / -, 768 878 / 220, 1,024 859 / 224, 1,536 835 / 229; 50,000 x
+// 50,000: 516, 514, 527 from 768 on).
+constexpr int UNG_TC_KEY_WINDOWS = 1024;
 constexpr int UNG_NARROW_CTAS_PER_SM = 2;
 constexpr int UNG_NARROW_PASS = 512;  // bank-2 windows a narrow CTA scores per pass
 }  // namespace plast

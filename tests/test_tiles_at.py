@@ -179,3 +179,29 @@ def test_callers_wide_costs_below_32(costs, slot, tile):  # noqa: F811
         wide_rests += goes_wide
         narrow_rests += not goes_wide
     assert wide_rests > 50 and narrow_rests > 50
+
+
+@pytest.mark.parametrize("s1", [31, 38])
+def test_key_by_key(costs, s1):  # noqa: F811
+    # one launch per key: a remainder beside full wide tiles is one more of
+    # them; without any, by the plain wide kernel's costs
+    c = dict(costs, wide_slot=0.140, wide_tile=3660.0)
+    B.plast_set_tile_costs(c)
+    B.plast_set_schedule(1)
+    n1, n2 = random_counts(np.random.default_rng(22))
+    k1, k2 = offsets(n1), offsets(n2)
+    tiles = B.plast_stage2_tiles(k1, k2, n_sms=152, s1=s1)
+    by_key = check_cover(tiles, k1, n1, n2)
+    assert (tiles[:, 4] == 0).all() and (tiles[:, 5] == n2[tiles[:, 0]]).all()
+    wide_rests = narrow_rests = 0
+    for k, t in by_key.items():
+        t = sorted(t)
+        if n1[k] >= T1:
+            assert [r for _, r, _ in t[:-1]] == [T1] * (len(t) - 1) and all(s == WIDE for _, _, s in t)
+            continue
+        wide = 0.317 * 128 * round_up(n2[k], 96) + 2960.0
+        goes_wide = narrow_cover(costs, int(n1[k]), n2[k]) >= wide
+        assert ([s for _, _, s in t] == [WIDE]) == goes_wide
+        wide_rests += goes_wide
+        narrow_rests += not goes_wide
+    assert wide_rests > 50 and narrow_rests > 50
