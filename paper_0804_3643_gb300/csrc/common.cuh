@@ -87,9 +87,13 @@ struct Tables {
 void build_tables(Tables* t);
 
 // Device copies (constant memory), filled once per device by upload_tables().
+// A file compiled as a whole program (it defines PLAST_WHOLE_PROGRAM) would get
+// zero-filled copies of its own, so it does not see them.
+#ifndef PLAST_WHOLE_PROGRAM
 extern __constant__ int8_t c_score[NCODE * NCODE];
 extern __constant__ int8_t c_cls2[NAA];
 extern __constant__ int8_t c_cls3[NAA];
+#endif
 
 // One byte from shared memory at a 32-bit shared address plus a constant
 // offset.  Issued as its own load so the byte goes through the load/store
@@ -121,12 +125,14 @@ inline plast_params resolve(const plast_params* p) {
 // Host: range of Section 4.2's filter threshold (0 = no filter).
 inline bool s0_ok(int32_t s0) { return s0 >= 0 && s0 <= 30000; }
 
+#ifndef PLAST_WHOLE_PROGRAM
 __device__ __forceinline__ int seed_key(int a0, int a1, int a2, int a3) {
   // Key = ((c1 * 2 + c2) * 11 + c3) * 20 + c4; -1 when a letter is a stop or
   // the sentinel.
   if ((a0 | a1 | a2 | a3) < 0 || a0 >= NAA || a1 >= NAA || a2 >= NAA || a3 >= NAA) return -1;
   return ((a0 * 2 + c_cls2[a1]) * 11 + c_cls3[a2]) * 20 + a3;
 }
+#endif
 
 }  // namespace plast
 

@@ -61,6 +61,7 @@
 // a quadrant instead of two 24.8; candidates queued by the epilogue warps
 // instead of masks decoded by the extend warps 22.4; tiles fetched by an
 // extend warp instead of one that runs ahead 22.7 (10,000 x 10,000: 4.0).
+#define PLAST_WHOLE_PROGRAM  // see build.py
 #include <atomic>
 
 #include "common.cuh"
