@@ -11,7 +11,8 @@ Prints one JSON line (rank 0).  ``value`` is ungapped pairs per second of the
 whole step with the banks' codes resident in device memory; ``e2e`` is the
 same metric with the codes copied from pinned host memory and the records
 copied back inside the timed region.  ``roofline`` rates the dominant kernel
-(stage 2) against the integer rate of its direct form; ``cpu_baseline`` times the CPU oracle
+(stage 2's wide tiles) against the fp4 tensor rate it is built on, and
+``direct_form`` its pace against extending every pair on the integer pipes; ``cpu_baseline`` times the CPU oracle
 on a bounded sample of the same workload.  ``--impl reference`` times the CPU
 oracle alone (the reference arm of this comparison).
 
@@ -44,6 +45,7 @@ CELLS_PER_CLK_SM = 128     # int16 cells per clock per SM on the ALU / FMA-heavy
 BAND_CELLS_PER_HIT = 2 * 64 * 17  # stage 3.1: two sides x LG rows x (2 x band + 1) columns
 MMA_FLOP_PER_PAIR = 27 * 64 * 2  # the tensor kernel's bound: 27 K steps of 64 a pair (two lay the base)
 FP4_PEAK_PFLOPS = 13.5     # nominal dense fp4 rate of the GPU
+KEY_WINDOWS = 1024         # per-key schedule: fewest bank-2 windows of a key on the tensor kernel
 ALU_LANES_PER_CLK_SM = 64  # ALU-pipe lanes per clock per SM (every integer max issues there)
 METRIC = "ungapped pairs/s and GCUPS at 1 GB300 (bit-exact), % of int/HBM roofline"
 
@@ -241,6 +243,42 @@ def committed_traffic():
     return t
 
 
+def stage2_roofline(tiles: np.ndarray, pairs: int, ms: float, persistent: bool, traffic) -> dict:
+    """Stage 2 rated by the MMA steps that the pairs of wide tiles take (their
+    bound on the fp4 tensor cores), over the time of both its kernels: the other
+    pairs add time and no steps.  tiles: the list that runs
+    (plast_stage2_tiles at the search's threshold)."""
+    t = tiles.astype(np.int64)
+    on_tensor = (t[:, 3] == 0) & (persistent | (t[:, 5] >= KEY_WINDOWS))
+    wide_pairs = int((t[:, 2] * (t[:, 5] - t[:, 4]))[on_tensor].sum())
+    achieved = wide_pairs * MMA_FLOP_PER_PAIR / (ms / 1e3) / 1e15
+    return {
+        "bound": "tensor",
+        "kernel": "stage 2: k_ungapped_mma (wide tiles: a bound on the fp4 tensor cores, the exact extension "
+                  "of the pairs it lets through), timed with the narrow tiles' kernel behind it",
+        "achieved": achieved, "peak": FP4_PEAK_PFLOPS, "unit": "PFLOP/s", "frac": achieved / FP4_PEAK_PFLOPS,
+        "traffic": traffic, "tensor_pairs": wide_pairs, "other_pairs": int(pairs) - wide_pairs, "kernel_ms": ms,
+        "peak_basis": f"nominal dense fp4 rate; {MMA_FLOP_PER_PAIR} FLOP a pair on the tensor cores",
+        "hbm_gbs": (traffic / (ms / 1e3) / 1e9) if traffic else None,
+    }
+
+
+def direct_form(pairs: int, ms: float, n_sm: int, sm_max: float) -> dict:
+    """Stage 2's pace against extending every pair on the integer pipes.  A
+    cell of that needs one int16 max (ALU pipe: 64 lanes x 2 halves per clock per
+    SM) and one int16 add (FMA-heavy pipe, the same rate): 128 cells per clock
+    per SM (the probe in paper_0804_3643_gb300/probe/pipes.cu measures the pipes).  The
+    tensor kernel extends only the pairs its bound lets through, so this is a
+    speed-up and no share of a bound."""
+    cells = pairs * CELLS_PER_PAIR / (ms / 1e3)
+    rate = n_sm * CELLS_PER_CLK_SM * sm_max * 1e6
+    return {
+        "cells_per_s": cells, "cells_per_pair": CELLS_PER_PAIR, "direct_cells_per_s": rate,
+        "speedup_over_direct_rate": cells / rate,
+        "basis": f"{n_sm} SMs x {CELLS_PER_CLK_SM} cells/clock x {sm_max:.0f} MHz (max SM clock)",
+    }
+
+
 def stage31_roofline(hits: int, ms: float, n_sm: int, sm_max: float, sm_mhz) -> dict:
     """Stage 3.1 against the integer ALU peak.  Unit: one band cell of the
     small gapped extension (2 sides x 64 rows x 17 columns per stage-2
@@ -324,6 +362,7 @@ def run_gpu(args, rank, world, local_rank):
     n_recs = recs.shape[0]
     del recs
     nb_gb = (g1.n_positions + g2.n_positions) * CELLS_PER_PAIR / 1e9
+    key_off = [B.plast_bank_export_index(g)[0].cpu().numpy() for g in (g1, g2)]
     g1.free()
     g2.free()
     torch.cuda.synchronize()
@@ -402,14 +441,7 @@ def run_gpu(args, rank, world, local_rank):
     sm_max = float(pk.get("sm_max_mhz", 2070.0))
     props = torch.cuda.get_device_properties(dev)
     n_sm = props.multi_processor_count
-    # The direct form's cell needs one int16 max (ALU pipe: 64 lanes x 2 halves
-    # per clock per SM) and one int16 add (FMA-heavy pipe, the same rate): 128
-    # cells per clock per SM (the probe in paper_0804_3643_gb300/probe/pipes.cu
-    # measures the pipes).  The wide tiles' kernel does not pay that for every
-    # pair: it bounds each pair's score on the fp4 tensor cores and extends the
-    # few that pass, so the fraction of this rate can exceed one.
-    peak_cells = n_sm * CELLS_PER_CLK_SM * sm_max * 1e6
-    achieved_cells = pairs * CELLS_PER_PAIR / (ung_ms / 1e3)
+    tile_list = B.plast_stage2_tiles(*key_off, n_sms=n_sm, s1=prm.s1)
     tr = committed_traffic()
     traffic = None
     if tr is not None:
@@ -437,27 +469,8 @@ def run_gpu(args, rank, world, local_rank):
         },
         "gcups": world * pairs * CELLS_PER_PAIR / (ms_step / 1e3) / 1e9,
         "stage_ms": stages,
-        "roofline": {
-            "bound": "alu",
-            "kernel": "stage 2: k_ungapped_mma (wide tiles: a bound on the fp4 tensor cores, the exact extension "
-                      "of the pairs it lets through) then k_ungapped_narrow (narrow tiles), timed together",
-            "achieved": achieved_cells / 1e12,
-            "peak": peak_cells / 1e12,
-            "unit": "Tcell/s",
-            "frac": achieved_cells / peak_cells,
-            "traffic": traffic,
-            "cells_per_pair": CELLS_PER_PAIR,
-            "kernel_ms": ung_ms,
-            "peak_basis": f"{n_sm} SMs x {CELLS_PER_CLK_SM} cells/clock (ALU pipe 64 lanes x 2 int16 halves for "
-                          f"the max, FMA-heavy pipe the same for the add) x {sm_max:.0f} MHz (max SM clock): the rate "
-                          "of extending every pair directly, which the tensor kernel does not do",
-            # (as if the narrow tiles' few per cent of the pairs went there too)
-            "tensor_pflops": pairs * MMA_FLOP_PER_PAIR / (ung_ms / 1e3) / 1e15,
-            "tensor_frac_of_nominal_fp4": pairs * MMA_FLOP_PER_PAIR / (ung_ms / 1e3) / 1e15 / FP4_PEAK_PFLOPS,
-            "frac_at_measured_clock": (achieved_cells / (n_sm * CELLS_PER_CLK_SM * clocks["sm_mhz"] * 1e6)
-                                       if clocks.get("sm_mhz") else None),
-            "hbm_gbs": (traffic / (ung_ms / 1e3) / 1e9) if traffic else None,
-        },
+        "roofline": stage2_roofline(tile_list, pairs, ung_ms, args.schedule == "persistent", traffic),
+        "direct_form": direct_form(pairs, ung_ms, n_sm, sm_max),
         "roofline_stage31": stage31_roofline(n_ung, gap_ms, n_sm, sm_max, clocks.get("sm_mhz")),
         "e2e": {"value": world * pairs / (e2e_ms / 1e3), "unit": "pairs/s", "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": int(rec_bytes), "ms_per_step": e2e_ms},
