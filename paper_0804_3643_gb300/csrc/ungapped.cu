@@ -128,13 +128,6 @@ __device__ __forceinline__ void unpack16(const uint4& p, uint32_t (&u)[8]) {
   u[7] = sext_pair(p.w, 1);
 }
 
-__device__ __forceinline__ void unpack8(uint32_t lo, uint32_t hi, uint32_t (&u)[4]) {
-  u[0] = sext_pair(lo, 0);
-  u[1] = sext_pair(lo, 1);
-  u[2] = sext_pair(hi, 0);
-  u[3] = sext_pair(hi, 1);
-}
-
 __device__ __forceinline__ void flush_warp(const uint64_t* wk, const uint32_t* wv, int n, int lane,
                                            unsigned long long* out_count, uint64_t* out_key, uint32_t* out_val,
                                            int64_t cap) {
