@@ -843,6 +843,9 @@ int plast_index_bank(const int8_t* codes, const int64_t* seq_off, int32_t n_seqs
   for (int32_t s = 0; s <= n_seqs; s++) b->h_pad_off[s] = h_off[s] + (int64_t)GAP * (s + 1);
 
   auto fail = [&](int rc) {
+    // (kernels already queued on st still use the bank's arrays, which are
+    // freed in order with another stream)
+    cudaStreamSynchronize(st);
     plast_bank_free(b);
     return rc;
   };
