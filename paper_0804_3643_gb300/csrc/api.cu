@@ -192,10 +192,15 @@ struct CostModel {
   int64_t wide_pass;  // bank-2 windows a CTA of the wide kernel scores per pass
   bool partial;       // the tensor kernel's: a wide tile that is not full costs less
   int64_t pass(int shape) const { return shape == UNG_WIDE ? wide_pass : (int64_t)UNG_NARROW_PASS; }
+  // n2 windows in whole passes (each by a constant: a plan asks some 20,000 times)
+  int64_t windows(int shape, int64_t n2) const {
+    if (shape != UNG_WIDE) return round_up(n2, UNG_NARROW_PASS);
+    return wide_pass == UNG_TC_PASS ? round_up(n2, UNG_TC_PASS) : round_up(n2, UNG_WIDE_PASS);
+  }
   // Slots a tile of `rows` rows is charged for (a partial wide tile of the
   // tensor kernel: a full one's share of what its passes cost).
   double slots(int shape, int64_t n2, int64_t rows) const {
-    const double full = (double)shape_rows(shape) * (double)round_up(n2, pass(shape));
+    const double full = (double)shape_rows(shape) * (double)windows(shape, n2);
     if (shape != UNG_WIDE || !partial) return full;
     return full * (double)(round_up(rows, 32) + TC_FIXED_ROWS) / (double)(UNG_T1 + TC_FIXED_ROWS);
   }
@@ -340,14 +345,16 @@ void build_tiles_from(const int64_t* ko1, const int64_t* ko2, bool largest_first
   if (largest_first) {
     // counting sort by decreasing n2 in steps that both kernels' passes are
     // multiples of: every tile cost rises with it; stable in key order
+    static_assert((UNG_NARROW_PASS & (UNG_NARROW_PASS - 1)) == 0, "the step is a power of two");
     const int64_t step = std::gcd(m.wide_pass, (int64_t)UNG_NARROW_PASS);
+    const int shift = __builtin_ctzll((unsigned long long)step);
     int64_t bmax = 0;
     for (const int k : keys) bmax = std::max<int64_t>(bmax, ko2[k + 1] - ko2[k]);
-    const int NB = (int)std::min<int64_t>(round_up(bmax, step) / step + 1, 1 << 20);
+    const int NB = (int)std::min<int64_t>(((bmax + step - 1) >> shift) + 1, 1 << 20);
     static thread_local std::vector<int32_t> count;
     count.assign((size_t)NB + 1, 0);
     auto bucket = [&](int k) {
-      const int64_t b = round_up(ko2[k + 1] - ko2[k], step) / step;
+      const int64_t b = (ko2[k + 1] - ko2[k] + step - 1) >> shift;
       return NB - 1 - (int)std::min<int64_t>(b, NB - 1);
     };
     for (const int k : keys) count[bucket(k) + 1]++;
