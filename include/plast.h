@@ -170,6 +170,9 @@ int plast_translate6(const uint8_t* dna, const int64_t* contig_off, int32_t n_co
  *           (device); total length < 2^31 - 2^26
  *   params  may be NULL (defaults)
  *   *out    receives the new bank (host)
+ * Device memory: 53 bytes a residue for the bank (48 of them the windows) and,
+ * until the last steps have run, 5 bytes a residue of stream-ordered scratch
+ * beside count tables of some megabytes.
  * The inputs are consumed before the call returns; the caller may free them
  * then.  The last steps (laying out the lists and windows) may still be running
  * on `stream` when the call returns: every later call that takes the bank
@@ -412,7 +415,9 @@ int plast_set_schedule(int mode);
  * variants and wide_stage_depth 0, 1 or 2).  plast_set_tile_shape forces the shape of every tile (1 wide;
  * 2, 3, 4, 5 narrow of 8, 4, 2, 16 rows; 0, the default, by cost).  Shapes change
  * the schedule, never the results.  Settings are process-wide and apply to
- * later calls.
+ * later calls.  (Planning keeps its lists with the thread that plans, 24 bytes a
+ * tile and 24 MB at most, until the thread ends: a plan that needed more gives
+ * them back.)
  */
 typedef struct plast_tile_costs {
   double wide_slot, wide_tile;       /* 128 rows */

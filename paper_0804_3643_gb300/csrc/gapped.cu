@@ -50,9 +50,9 @@
 // 0): it never raises the best value, and the end column is looked for on the
 // grid only.
 //
-// Bound by the rate of three-operand instructions: of 13.3 instructions a
+// Bound by the rate of three-operand instructions: of 13.4 instructions a
 // cell 9 read three registers, and a loop of the same mix on registers alone
-// takes 17.3 clocks a cell per warp and scheduler where this takes 18.1.
+// takes 17.3 clocks a cell per warp and scheduler where this takes 17.4.
 // Four rows share their B offsets in registers, and all 64 rows run through
 // one loop of four (15 KB of code; eight rows unrolled do not fit the
 // instruction cache: 23.3 ms, two rows move more registers: 19.5): 18.6 ms for

@@ -294,8 +294,9 @@ struct SplitSmem {
 static_assert(IX_CHUNK <= 1 << 14 && NKEYS <= 1 << 14, "packing");
 static_assert(sizeof(SplitSmem) <= 48 * 1024, "static shared memory");
 
-// Waits on shared memory, one chunk a CTA and three CTAs an SM (four: 1.00 ms
-// for 0.98 at 206 M positions, their 32 registers spill).
+// Bound by the ALU pipe (89 % busy, the ballots' selects; issue 65 %), one chunk
+// a CTA and three CTAs an SM (four: 1.00 ms for 0.98 at 206 M positions, their
+// 32 registers spill).
 __global__ void __launch_bounds__(IX_THREADS, 3) k_index_split(const int8_t* pad, int64_t n_pad, IndexShape sh,
                                                                const int64_t* off, uint32_t* by_pos,
                                                                uint8_t* by_lo) {

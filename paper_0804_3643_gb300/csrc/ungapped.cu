@@ -13,9 +13,9 @@
 //
 // Two tile shapes, each in its own persistent kernel (k_ungapped<N16>,
 // k_ungapped_narrow), launched one after the other over the work list:
-//  * wide: up to 128 rows (at thresholds below UNG_TC_MIN_S1; above it wide
-//    tiles run on the tensor cores, ungapped_mma.cu, which scores most pairs
-//    by a bound only).  Lane (g, js) of a warp scores bank-2 window js
+//  * wide: up to 128 rows (at thresholds below UNG_TC_MIN_S1 and, key by key,
+//    lists below UNG_TC_KEY_WINDOWS; the others run on the tensor cores,
+//    ungapped_mma.cu, which scores most pairs by a bound only).  Lane (g, js) of a warp scores bank-2 window js
 //    (4 per warp) against rows 16g .. 16g+15; the 8 lanes of a window read
 //    one 128-byte profile row per cell, so a warp's loads come out of shared
 //    memory in the minimum number of wavefronts.  Two refinements:
